@@ -1026,6 +1026,10 @@ struct LevelTables {
   std::vector<int> blk, bblk, fblk, cs;
 };
 
+// Levels a hierarchy can have: every level halves an extent of some part, and
+// a part's extents multiply to less than 2^31.
+constexpr int kMaxLevels = 128;
+
 // The host side of a level's tables: part descriptors (L.dparts), tile and
 // brick decomposition, operator-apply shape.  Copies nothing.
 void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
@@ -1168,6 +1172,29 @@ void upload_levels(ssamg_solver s, cudaStream_t st) {
     L.d_cellstart = (int*)put(t[l].cs.data(), sizeof(int) * (np + 1));
   }
   SSAMG_CUDA(cudaMemcpyAsync(dev, s->h_up, o, cudaMemcpyHostToDevice, st));
+}
+
+// The row-job form of every level (see u_row_job), from its longest coupling
+// row: rows of more than two entries per lane go to the entry-balanced form.
+// Measured (8 parts of 64^3, FP32 cycle, restriction onto / prolongation from
+// the level): 131,072 cells, mean row 8, longest 45, 16 lanes: 7.7 -> 6.7 and
+// 6.4 -> 4.1 us; 32,768 cells, mean 11, longest 93: 7.2 -> 4.1 and 6.1 -> 3.3
+// us.  Two parts with refinement, longest row 25 on 16 lanes: 2.0 -> 2.6 us, so
+// the lanes stay below the line.  Larger levels have rows enough to hide the
+// long ones, and lose: 524,288 cells FP32 10.0 -> 8.4 and 6.4 -> 7.4 us; FP64
+// 65,536 cells 10.0 -> 11.5 and 8.4 -> 10.0 us, 32,768 cells 9.5 -> 9.7 and 7.9
+// -> 7.2 us, 16,384 cells 10.8 -> 7.4 and 7.9 -> 5.1 us.
+void row_job_blocks(ssamg_solver s, const int* maxrow, cudaStream_t st) {
+  bool any = false;
+  const long long most = s->prm.precision == 1 ? SSAMG_UROW_CELLS_F32 : SSAMG_UROW_CELLS_F64;
+  for (size_t l = 0; l < s->lev.size(); ++l) {
+    Level& L = s->lev[l];
+    if (L.nr == 0 || L.nnz == 0 || L.N > most || maxrow[l] <= 2 * L.tpr) continue;
+    L.nublk = (int)cdivll(L.nnz, SSAMG_UROW_ENTRIES);
+    L.u_rb = aalloc<int4>(s->arena, L.nublk);
+    any = true;
+  }
+  if (any) launch_urb(s->lev, st);
 }
 
 // Coarse-level transition run by one cluster (see kernels_tail.cu): picks the
@@ -1317,7 +1344,7 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
     s->h_int = nullptr;
     s->h_dbl = nullptr;
     s->h_sc = pinned_new<PcgScalars>(s->nprob);
-    s->h_int = pinned_new<int>(16);
+    s->h_int = pinned_new<int>(4 + kMaxLevels);
     s->h_dbl = pinned_new<double>(2 * s->nprob + 16);
     s->h_cap = s->nprob;
   }
@@ -1560,8 +1587,9 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   for (int l = 1; l <= Lc; ++l) maxN = std::max(maxN, s->lev[l].N);
   int* marker = nullptr;
   int* scan_tmp = nullptr;
-  s->d_err = aalloc<int>(s->arena, 4);
-  SSAMG_CUDA(cudaMemsetAsync(s->d_err, 0, sizeof(int) * 4, st));
+  // 4 status words, then the longest coupling row of every level
+  s->d_err = aalloc<int>(s->arena, 4 + Lc + 1);
+  SSAMG_CUDA(cudaMemsetAsync(s->d_err, 0, sizeof(int) * (4 + Lc + 1), st));
   // The coupling rows of a coarse level are fixed by the structure alone
   // (which coarse cells the fine coupling rows' P rows reach), so they are
   // found one level ahead: each level waits on the host once, for the entry
@@ -1728,6 +1756,7 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
           base += al(sizeof(float) * L.N);
         }
       }
+      launch_urow_max(s->lev, s->d_err + 4, st);
     }
   }
 
@@ -1807,10 +1836,11 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
       }
     }
   }
-  SSAMG_CUDA(cudaMemcpyAsync(s->h_int, s->d_err, sizeof(int) * 4, cudaMemcpyDeviceToHost, st));
+  SSAMG_CUDA(cudaMemcpyAsync(s->h_int, s->d_err, sizeof(int) * (4 + Lc + 1), cudaMemcpyDeviceToHost, st));
   SSAMG_CUDA(cudaStreamSynchronize(st));
   if (s->h_int[0]) throw SsamgError{SSAMG_ERR_UNSUPPORTED, "a coarse coupling row has more than 1024 candidates"};
   if (s->h_int[2]) throw SsamgError{SSAMG_ERR_BREAKDOWN, "coarsest operator is not positive definite"};
+  row_job_blocks(s, s->h_int + 4, st);
   // ---- coarse-level transition in one cluster (use_tail = 3)
   s->ctail_lt = -1;
   if (s->prm.use_tail == 3) {

@@ -17,9 +17,9 @@
 // The same tiles with the SSAMG_CPT_LARGE steps unrolled and predicated, so
 // that a thread issues the loads of all its cells before it consumes the
 // first; for kernels light enough in registers (restriction, prolongation).
-#define TILE_LOOP_UNROLLED(c, P)                                                           \
+#define TILE_LOOP_UNROLLED(c, P, B)                                                        \
   _Pragma("unroll") for (int c##_m = 0; c##_m < SSAMG_CPT_LARGE; ++c##_m)                  \
-    if (const int c = ((int)blockIdx.x - (P).blk0) * (P).cpt * SSAMG_BLOCK +               \
+    if (const int c = ((B) - (P).blk0) * (P).cpt * SSAMG_BLOCK +                           \
                       (int)threadIdx.x + c##_m * SSAMG_BLOCK;                              \
         c##_m < (P).cpt && c < (P).ncell)
 #define TILE_LOOP_FINE(c, P)                                                               \
@@ -509,13 +509,86 @@ __device__ __forceinline__ void u_row_sum(const LevelView<T>& L, int r, int l4, 
   if (r < L.nr && l4 == 0) L.uy[L.u_rows[r]] = acc;
 }
 
-// Row job of a launch: block rb's threads take SSAMG_BLOCK / L.tpr rows,
-// L.tpr lanes each (all threads must call; waits for the predecessor inside).
-template <class T, class Pre, class F>
+// Row job of a launch: U x of the rows of row-job block rb (all threads must
+// call; waits for the predecessor inside).  f and pre() are as in u_row_sum.
+// Two forms, the same sums bit for bit (a row's entries strided over L.tpr
+// lanes, then the shuffle tree), chosen per level at setup from its longest
+// row (see row_job_blocks in abi.cu; a template argument, so that the lane
+// form's kernels keep their registers and L1):
+//   EB = false: block rb takes SSAMG_BLOCK / L.tpr rows, L.tpr lanes each;
+//     a lane loads its row's entries one after another.
+//   EB = true (L.u_rb set): the blocks hold equal numbers of entries (SSAMG_UROW_ENTRIES,
+//     to the end of the last row), a thread per entry: its setup data is
+//     loaded before the wait, and after it every entry's value is one round of
+//     gathers, handed to the row's lanes through shared memory.  For levels
+//     with long rows (parts coarsened along different directions: 62 entries
+//     in the longest hundredth of the rows, median 6), where the longest row's
+//     dependent loads set the kernel's time: restriction onto a 32,768-cell
+//     level of 8 parts with 103,356 entries 6.9 -> 3.8 us, prolongation from
+//     it 6.1 -> 2.6 us; levels of short rows are faster with the lanes (one
+//     barrier less: 2.0 vs 2.6 us with rows of at most 25 entries).
+template <bool EB, class T, class Pre, class F>
 __device__ __forceinline__ void u_row_job(const LevelView<T>& L, int rb, Pre&& pre, F&& f) {
+  const int t = threadIdx.x;
   const int sh = __ffs(L.tpr) - 1;  // tpr is a power of two
-  u_row_sum<true>(L, rb * (SSAMG_BLOCK >> sh) + ((int)threadIdx.x >> sh),
-                  (int)threadIdx.x & (L.tpr - 1), pre, f);
+  const int sub = t >> sh, lane = t & (L.tpr - 1), ngrp = SSAMG_BLOCK >> sh;
+  if constexpr (!EB) {
+    u_row_sum<true>(L, rb * ngrp + sub, lane, pre, f);
+    return;
+  } else {
+    constexpr int CAP = SSAMG_UROW_SLOTS * SSAMG_BLOCK;
+    __shared__ T su[CAP], sx[CAP];
+    __shared__ int3 srow[SSAMG_BLOCK];  // entry range and cell of the block's rows
+    const int4 blk = L.u_rb[rb];
+    const int r0 = blk.x, nrows = blk.y, e0 = blk.z, e1 = blk.w;
+    // (entries beyond the slots: a row of more than SSAMG_UROW_ENTRIES; more
+    // rows than threads: rows without entries)
+    if (nrows > SSAMG_BLOCK || e1 - e0 > CAP) {
+      pdl_wait();
+      for (int b = 0; b < nrows; b += ngrp)
+        u_row_sum<false>(L, b + sub < nrows ? r0 + b + sub : L.nr, lane, pre, f);
+      return;
+    }
+    if (t < nrows)
+      srow[t] = make_int3(L.u_ptr[r0 + t] - e0, L.u_ptr[r0 + t + 1] - e0, L.u_rows[r0 + t]);
+    int c[SSAMG_UROW_SLOTS];
+    decltype(pre(0, 0)) s[SSAMG_UROW_SLOTS];
+  #pragma unroll
+    for (int m = 0; m < SSAMG_UROW_SLOTS; ++m) {
+      const int q = e0 + t + m * SSAMG_BLOCK;
+      if (q < e1) {
+        c[m] = L.u_col[q];
+        su[t + m * SSAMG_BLOCK] = L.u_val[q];
+        s[m] = pre(c[m], q);
+      }
+    }
+    pdl_wait();
+    T v[SSAMG_UROW_SLOTS];
+  #pragma unroll
+    for (int m = 0; m < SSAMG_UROW_SLOTS; ++m) {
+      const int q = e0 + t + m * SSAMG_BLOCK;
+      if (q < e1) v[m] = f(c[m], q, s[m]);
+    }
+  #pragma unroll
+    for (int m = 0; m < SSAMG_UROW_SLOTS; ++m)
+      if (e0 + t + m * SSAMG_BLOCK < e1) sx[t + m * SSAMG_BLOCK] = v[m];
+    __syncthreads();
+    for (int b = 0; b < nrows; b += ngrp) {
+      const int rr = b + sub;
+      const int3 row = rr < nrows ? srow[rr] : make_int3(0, 0, 0);
+      T acc = (T)0;
+      for (int q = row.x + lane; q < row.y; q += L.tpr) acc = fma(su[q], sx[q], acc);
+      for (int o = 1; o < L.tpr; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (rr < nrows && lane == 0) L.uy[row.z] = acc;
+    }
+  }
+}
+
+// The role of a block of a launch with nu row-job blocks, tile0 of the other
+// blocks before them: a row-job block below nu, else nu plus the tile.
+__device__ __forceinline__ int row_job_role(int nu, int tile0) {
+  const int v = (int)blockIdx.x - tile0;
+  return v < 0 ? v + (int)gridDim.x : v;
 }
 
 // Block-wide sum (deterministic: fixed order).  sh holds NT doubles.  The

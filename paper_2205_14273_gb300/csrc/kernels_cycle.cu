@@ -21,15 +21,17 @@ __global__ void k_relax0(int N, const T* dinv, const T* b,
   if (g < N) x[g] = dinv[g] * b[g];
 }
 
-// x = omega M^-1 b on blocks [0, nb); row jobs uy = U x on the rest.  The
+// x = omega M^-1 b, and uy = U x on nu row-job blocks (after tile0 of the
+// others, here and below, see row_job_role).  The
 // diagonal (setup data) is fetched before the wait for the predecessor.
-template <class T>
-__global__ void __launch_bounds__(NT) k_relax0_u(LevelView<T> L, int nb, const T* b,
+template <class T, bool EB>
+__global__ void __launch_bounds__(NT) k_relax0_u(LevelView<T> L, int nu, int tile0, const T* b,
                                                  T* x) {
   pdl_trigger();
-  if ((int)blockIdx.x < nb) {
+  const int role = row_job_role(nu, tile0);
+  if (role >= nu) {
     // SSAMG_EW cells per thread, strided by the block: all loads in flight
-    const int g0 = blockIdx.x * (NT * SSAMG_EW) + threadIdx.x;
+    const int g0 = (role - nu) * (NT * SSAMG_EW) + threadIdx.x;
     T d[SSAMG_EW];
 #pragma unroll
     for (int m = 0; m < SSAMG_EW; ++m) d[m] = g0 + m * NT < L.N ? L.dinv[g0 + m * NT] : (T)0;
@@ -39,20 +41,21 @@ __global__ void __launch_bounds__(NT) k_relax0_u(LevelView<T> L, int nb, const T
       if (g0 + m * NT < L.N) x[g0 + m * NT] = d[m] * b[g0 + m * NT];
     return;
   }
-  u_row_job(
-      L, blockIdx.x - nb, [&](int col, int) { return L.dinv[col]; },
+  u_row_job<EB>(
+      L, role, [&](int col, int) { return L.dinv[col]; },
       [&](int col, int, T d) { return d * b[col]; });
 }
 
 // First pre-relaxation of the cycle straight from the FP64 PCG residual:
-// b0 = (T) r, x = omega M^-1 b0 on the cell blocks; uy = U x on the rest.
-template <class T>
-__global__ void __launch_bounds__(NT) k_relax0_u_first(LevelView<T> L, int nb,
+// b0 = (T) r, x = omega M^-1 b0 on the cell blocks; uy = U x on the row-job blocks.
+template <class T, bool EB>
+__global__ void __launch_bounds__(NT) k_relax0_u_first(LevelView<T> L, int nu, int tile0,
                                                        const double* r64,
                                                        T* b0, T* x) {
   pdl_trigger();
-  if ((int)blockIdx.x < nb) {
-    const int g0 = blockIdx.x * (NT * SSAMG_EW) + threadIdx.x;
+  const int role = row_job_role(nu, tile0);
+  if (role >= nu) {
+    const int g0 = (role - nu) * (NT * SSAMG_EW) + threadIdx.x;
     T d[SSAMG_EW];
 #pragma unroll
     for (int m = 0; m < SSAMG_EW; ++m) d[m] = g0 + m * NT < L.N ? L.dinv[g0 + m * NT] : (T)0;
@@ -68,16 +71,16 @@ __global__ void __launch_bounds__(NT) k_relax0_u_first(LevelView<T> L, int nb,
     }
     return;
   }
-  u_row_job(
-      L, blockIdx.x - nb, [&](int col, int) { return L.dinv[col]; },
+  u_row_job<EB>(
+      L, role, [&](int col, int) { return L.dinv[col]; },
       [&](int col, int, T d) { return d * (T)r64[col]; });
 }
 
 // uy = U x (row jobs only)
-template <class T>
+template <class T, bool EB>
 __global__ void __launch_bounds__(NT) k_uy(LevelView<T> L, const T* x) {
   pdl_trigger();
-  u_row_job(
+  u_row_job<EB>(
       L, blockIdx.x, [](int, int) { return 0; }, [&](int col, int, int) { return x[col]; });
 }
 
@@ -476,18 +479,19 @@ struct RCol {
 
 // bc = P^T r, one coarse cell per thread: the anchor (weight 1) and the two
 // fine points beside it along d* (weights PE of the west one, PW of the east).
-template <class T>
+template <class T, bool EB>
 __global__ void __launch_bounds__(NT) k_restrict(LevelView<T> F, LevelView<T> C,
-                                                 const T* r, T* bc, T* xc, int nb) {
+                                                 const T* r, T* bc, T* xc, int nu, int tile0) {
   pdl_trigger();
   __shared__ DPart fp;
   __shared__ DPart cp;
-  if ((int)blockIdx.x >= nb) {
+  const int role = row_job_role(nu, tile0);
+  if (role < nu) {
     // row jobs of the coarse level's pre-relaxation: uy = U x with
     // x = omega M^-1 b at each coupling's column, b rebuilt there from the
     // column's restriction row exactly as the tiles compute it
-    u_row_job(
-        C, blockIdx.x - nb,
+    u_row_job<EB>(
+        C, role,
         [&](int col, int q) {
           return RCol<T>{C.u_rj[3 * q], C.u_rj[3 * q + 1], C.u_rj[3 * q + 2], C.u_rw[2 * q],
                          C.u_rw[2 * q + 1], C.dinv[col]};
@@ -500,12 +504,13 @@ __global__ void __launch_bounds__(NT) k_restrict(LevelView<T> F, LevelView<T> C,
         });
     return;
   }
-  int p = block_part(C.blk, C.parts, C.np, cp);
+  const int tile = role - nu;
+  int p = block_part(C.blk, C.parts, C.np, cp, tile);
   part_of(F.parts, p, fp);
   __syncthreads();
   pdl_wait();
   if (C.skip && C.skip[cp.prob].done) return;  // problem already stopped
-  TILE_LOOP_UNROLLED(cc, cp) {
+  TILE_LOOP_UNROLLED(cc, cp, tile) {
     int I[3];
     cell_coords(cp, cc, I[0], I[1], I[2]);
     const int d = fp.dstar;
@@ -557,9 +562,9 @@ constexpr int RP_Z = SSAMG_BRICK_Z;
 // The thread's column (i, j) and first z of its brick; false when the column
 // lies outside the part.  The brick's position comes from shared memory,
 // decoded once per block (bpos[0..2], written by thread 0 of the block).
-__device__ __forceinline__ void rp_brick_origin(const DPart& sp, int* bpos) {
+__device__ __forceinline__ void rp_brick_origin(const DPart& sp, int brick, int* bpos) {
   if (threadIdx.x == 0) {
-    const int bl = (int)blockIdx.x - sp.bblk0;
+    const int bl = brick - sp.bblk0;
     bpos[0] = bl % sp.bb[0];
     const int byz = bl / sp.bb[0];
     bpos[1] = byz % sp.bb[1];
@@ -643,16 +648,17 @@ __device__ __forceinline__ void restrict_column(const LevelView<T>& F, const Lev
   }
 }
 
-template <class T>
+template <class T, bool EB>
 __global__ void __launch_bounds__(NT) k_restrict_b(LevelView<T> F, LevelView<T> C, const T* r,
-                                                   T* bc, T* xc, int nb) {
+                                                   T* bc, T* xc, int nu, int tile0) {
   pdl_trigger();
   __shared__ DPart fp;
   __shared__ DPart cp;
   __shared__ int bpos[3];
-  if ((int)blockIdx.x >= nb) {
-    u_row_job(
-        C, blockIdx.x - nb,
+  const int role = row_job_role(nu, tile0);
+  if (role < nu) {
+    u_row_job<EB>(
+        C, role,
         [&](int col, int q) {
           return RCol<T>{C.u_rj[3 * q], C.u_rj[3 * q + 1], C.u_rj[3 * q + 2], C.u_rw[2 * q],
                          C.u_rw[2 * q + 1], C.dinv[col]};
@@ -665,10 +671,11 @@ __global__ void __launch_bounds__(NT) k_restrict_b(LevelView<T> F, LevelView<T> 
         });
     return;
   }
-  const int p = block_part(C.bblk, C.parts, C.np, cp);
+  const int brick = role - nu;
+  const int p = block_part(C.bblk, C.parts, C.np, cp, brick);
   part_of(F.parts, p, fp);
   __syncthreads();
-  rp_brick_origin(cp, bpos);
+  rp_brick_origin(cp, brick, bpos);
   __syncthreads();
   int I0, I1, K0;
   const bool ok = rp_column(cp, bpos, I0, I1, K0);
@@ -763,15 +770,16 @@ __device__ __forceinline__ void prolong_column(const LevelView<T>& F, const DPar
   }
 }
 
-template <class T>
+template <class T, bool EB>
 __global__ void __launch_bounds__(NT) k_prolong_ub(LevelView<T> F, const T* ec, const T* xin,
-                                                   T* xout, int nb) {
+                                                   T* xout, int nu, int tile0) {
   pdl_trigger();
   __shared__ DPart fp;
   __shared__ int bpos[3];
-  if ((int)blockIdx.x >= nb) {
-    u_row_job(
-        F, blockIdx.x - nb,
+  const int role = row_job_role(nu, tile0);
+  if (role < nu) {
+    u_row_job<EB>(
+        F, role,
         [&](int, int q) {
           return PCol<T>{F.u_pj[2 * q], F.u_pj[2 * q + 1], F.u_pw[2 * q], F.u_pw[2 * q + 1]};
         },
@@ -784,19 +792,14 @@ __global__ void __launch_bounds__(NT) k_prolong_ub(LevelView<T> F, const T* ec, 
     return;
   }
   // two blocks per brick: block b takes the half (b & 1) of brick b >> 1
-  block_part(F.bblk, F.parts, F.np, fp, (int)blockIdx.x >> 1);
+  const int half = role - nu;
+  block_part(F.bblk, F.parts, F.np, fp, half >> 1);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    const int bl = ((int)blockIdx.x >> 1) - fp.bblk0;
-    bpos[0] = bl % fp.bb[0];
-    const int byz = bl / fp.bb[0];
-    bpos[1] = byz % fp.bb[1];
-    bpos[2] = byz / fp.bb[1];
-  }
+  rp_brick_origin(fp, half >> 1, bpos);
   __syncthreads();
   int i, j, k0;
   const bool ok = rp_column(fp, bpos, i, j, k0);
-  k0 += ((int)blockIdx.x & 1) * PZ;
+  k0 += (half & 1) * PZ;
   const int kend = min(k0 + PZ, fp.n[2]);
   if (!ok) {
     pdl_wait();
@@ -815,15 +818,16 @@ __global__ void __launch_bounds__(NT) k_prolong_ub(LevelView<T> F, const T* ec, 
 // coupling's column is rebuilt from xin and the column's P row (precomputed
 // at setup), so the two roles need no ordering.  P rows are setup data and
 // are fetched before the wait for the predecessor.
-template <class T>
+template <class T, bool EB>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 8 : 6) k_prolong_u(LevelView<T> F, const T* ec,
                                                   const T* xin, T* xout,
-                                                  int nb) {
+                                                  int nu, int tile0) {
   pdl_trigger();
   __shared__ DPart fp;
-  if ((int)blockIdx.x >= nb) {
-    u_row_job(
-        F, blockIdx.x - nb,
+  const int role = row_job_role(nu, tile0);
+  if (role < nu) {
+    u_row_job<EB>(
+        F, role,
         [&](int, int q) {
           return PCol<T>{F.u_pj[2 * q], F.u_pj[2 * q + 1], F.u_pw[2 * q], F.u_pw[2 * q + 1]};
         },
@@ -835,10 +839,11 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 8 : 6) k_prolong_u(LevelV
         });
     return;
   }
-  int p = block_part(F.blk, F.parts, F.np, fp);
+  const int tile = role - nu;
+  int p = block_part(F.blk, F.parts, F.np, fp, tile);
   __syncthreads();
   // the first tile cell's P row (setup data) is fetched before the wait
-  const int cfirst = ((int)blockIdx.x - fp.blk0) * fp.cpt * SSAMG_BLOCK + (int)threadIdx.x;
+  const int cfirst = (tile - fp.blk0) * fp.cpt * SSAMG_BLOCK + (int)threadIdx.x;
   PRow<T> pr0{-1, -1, (T)0, (T)0};
   if (cfirst < fp.ncell) {
     int i, j, k;
@@ -847,7 +852,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 8 : 6) k_prolong_u(LevelV
   }
   pdl_wait();
   if (F.skip && F.skip[fp.prob].done) return;  // problem already stopped
-  TILE_LOOP_UNROLLED(c, fp) {
+  TILE_LOOP_UNROLLED(c, fp, tile) {
     PRow<T> pr = pr0;
     if (c != cfirst) {
       int i, j, k;
@@ -1627,6 +1632,14 @@ bool uses_bricks(const Level& L) {
 const int* partial_ranges(const Level& L, const PcgCtx& c) { return uses_bricks(L) ? c.pbb : c.pb; }
 const int* final_ranges(const Level& L, const PcgCtx& c) { return uses_bricks(L) ? c.pbb : c.pb; }
 
+// Blocks of a launch with nt tile blocks that come before its row jobs.  The
+// entry-balanced row jobs (levels of long rows) go first: their chain of
+// dependent loads is the longer one and the tiles run beside it (restriction
+// onto a 131,072-cell level 7.9 -> 6.7 us).  The lane form has many more blocks
+// and would hold up the tiles of a large level (1M cells: 10.0 us after the
+// tiles, 13.1 us before them).
+static int row_job_tile0(const Level& L, int nt) { return L.u_rb ? 0 : nt; }
+
 template <class T>
 void launch_relax0(const Level& L, const T* b, T* x, cudaStream_t st) {
   const T* dinv = L.view<T>().dinv;
@@ -1636,7 +1649,7 @@ void launch_relax0(const Level& L, const T* b, T* x, cudaStream_t st) {
 template <class T>
 void launch_relax0_u(const Level& L, const T* b, T* x, cudaStream_t st) {
   int nb = cdiv(L.N, NT * SSAMG_EW);
-  launch_k(k_relax0_u<T>, nb + L.nublk, NT, 0, st, L.view<T>(), nb, b, x);
+  launch_k(L.u_rb ? k_relax0_u<T, true> : k_relax0_u<T, false>, nb + L.nublk, NT, 0, st, L.view<T>(), L.nublk, row_job_tile0(L, nb), b, x);
   SSAMG_LAUNCH_CHECK();
 }
 // one group of g right-hand sides (g = 1 .. SSAMG_RHS_GROUP) of shape SHC
@@ -1660,7 +1673,8 @@ void launch_relax0_u(const Level& L, const T* b, T* x, cudaStream_t st) {
 template <class T>
 void launch_relax0_u_first(const Level& L, const double* r64, T* b0, T* x, cudaStream_t st) {
   int nb = cdiv(L.N, NT * SSAMG_EW);
-  launch_k(k_relax0_u_first<T>, nb + L.nublk, NT, 0, st, L.view<T>(), nb, r64, b0, x);
+  launch_k(L.u_rb ? k_relax0_u_first<T, true> : k_relax0_u_first<T, false>, nb + L.nublk, NT, 0, st, L.view<T>(), L.nublk,
+           row_job_tile0(L, nb), r64, b0, x);
   SSAMG_LAUNCH_CHECK();
 }
 template <class T>
@@ -1680,17 +1694,18 @@ void launch_relax_final(const Level& L, const T* x, const T* b, double* z, const
 template <class T>
 void launch_prolong_u(const Level& F, const T* ec, const T* xin, T* xout, cudaStream_t st) {
   if (rp_bricks(F)) {
-    launch_k(k_prolong_ub<T>, 2 * F.nbblk + F.nublk, NT, 0, st, F.view<T>(), ec, xin, xout,
-             2 * F.nbblk);
+    launch_k(F.u_rb ? k_prolong_ub<T, true> : k_prolong_ub<T, false>, 2 * F.nbblk + F.nublk, NT, 0, st, F.view<T>(), ec, xin, xout,
+             F.nublk, row_job_tile0(F, 2 * F.nbblk));
   } else {
-    launch_k(k_prolong_u<T>, F.nblk + F.nublk, NT, 0, st, F.view<T>(), ec, xin, xout, F.nblk);
+    launch_k(F.u_rb ? k_prolong_u<T, true> : k_prolong_u<T, false>, F.nblk + F.nublk, NT, 0, st, F.view<T>(), ec, xin, xout, F.nublk,
+             row_job_tile0(F, F.nblk));
   }
   SSAMG_LAUNCH_CHECK();
 }
 template <class T>
 void launch_uy(const Level& L, const T* x, cudaStream_t st) {
   if (L.nublk == 0) return;
-  launch_k(k_uy<T>, L.nublk, NT, 0, st, L.view<T>(), x);
+  launch_k(L.u_rb ? k_uy<T, true> : k_uy<T, false>, L.nublk, NT, 0, st, L.view<T>(), x);
   SSAMG_LAUNCH_CHECK();
 }
 
@@ -1768,11 +1783,11 @@ void launch_restrict(const Level& F, const Level& Cl, const T* r, T* bc, T* xc, 
   // with xc: also x = omega M^-1 b on the coarse level, and its U x row jobs
   const int nrow = xc ? Cl.nublk : 0;
   if (rp_bricks(Cl)) {
-    launch_k(k_restrict_b<T>, Cl.nbblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc,
-             Cl.nbblk);
+    launch_k(Cl.u_rb ? k_restrict_b<T, true> : k_restrict_b<T, false>, Cl.nbblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc,
+             nrow, row_job_tile0(Cl, Cl.nbblk));
   } else {
-    launch_k(k_restrict<T>, Cl.nblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc,
-             Cl.nblk);
+    launch_k(Cl.u_rb ? k_restrict<T, true> : k_restrict<T, false>, Cl.nblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc,
+             nrow, row_job_tile0(Cl, Cl.nblk));
   }
   SSAMG_LAUNCH_CHECK();
 }

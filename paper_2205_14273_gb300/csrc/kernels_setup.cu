@@ -926,6 +926,52 @@ __global__ void k_ucols(LevelView<double> Fp, LevelView<double> L, long long nnz
   if (rj) urcol(Fp, L, q, rj, rw, rw32);
 }
 
+// The rows of every row-job block: block k of a level takes the rows whose
+// entries start in [k E, (k + 1) E), E = SSAMG_UROW_ENTRIES (two binary
+// searches over u_ptr; setup data, so that the solve's row jobs read their
+// range with one load).
+struct UrbLevel {
+  const int* u_ptr;
+  int4* u_rb;
+  int nr, t0;
+  int* maxrow;
+};
+struct UrbArgs {
+  int nl, n;
+  UrbLevel lv[SSAMG_DINV_LEVELS];
+};
+__global__ void __launch_bounds__(NT) k_urb(const __grid_constant__ UrbArgs A) {
+  const int t = blockIdx.x * NT + threadIdx.x;
+  if (t >= A.n) return;
+  int l = 0;
+  while (l + 1 < A.nl && t >= A.lv[l + 1].t0) ++l;
+  const UrbLevel& L = A.lv[l];
+  // first row whose entries start at e or later (nr: none)
+  auto first = [&](int e) {
+    int lo = 0, hi = L.nr;
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (L.u_ptr[mid] >= e) hi = mid; else lo = mid + 1;
+    }
+    return lo;
+  };
+  const int k = t - L.t0;
+  const int r0 = first(k * SSAMG_UROW_ENTRIES), r1 = first((k + 1) * SSAMG_UROW_ENTRIES);
+  L.u_rb[k] = make_int4(r0, r1 - r0, L.u_ptr[r0], L.u_ptr[r1]);
+}
+
+// The longest U row of every level: a thread per row, a warp's maximum per
+// atomic.
+__global__ void __launch_bounds__(NT) k_urow_max(const __grid_constant__ UrbArgs A) {
+  int l = 0;
+  while (l + 1 < A.nl && (int)blockIdx.x * NT >= A.lv[l + 1].t0) ++l;
+  const UrbLevel& L = A.lv[l];  // levels start at block boundaries
+  const int r = (int)blockIdx.x * NT + (int)threadIdx.x - L.t0;
+  const int n = r < L.nr ? L.u_ptr[r + 1] - L.u_ptr[r] : 0;
+  const int m = __reduce_max_sync(0xffffffffu, n);
+  if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(L.maxrow, m);
+}
+
 // ---------------------------------------------------------------------------
 // K5: diagonal of omega M^-1 (Section 3.4).
 // ---------------------------------------------------------------------------
@@ -1413,6 +1459,38 @@ void launch_ucols(const Level* Fp, const Level& L, bool fp32, bool pj, bool rj, 
   SSAMG_LAUNCH_CHECK();
 }
 
+
+void launch_urow_max(const std::vector<Level>& lev, int* maxrow, cudaStream_t st) {
+  const int nlev = (int)lev.size();
+  for (int l = 0; l < nlev;) {
+    UrbArgs a{};
+    for (; l < nlev && a.nl < SSAMG_DINV_LEVELS; ++l) {
+      const Level& L = lev[l];
+      if (L.nr == 0 || L.nnz == 0) continue;
+      a.lv[a.nl++] = UrbLevel{L.u_ptr, nullptr, L.nr, a.n, maxrow + l};
+      a.n += cdiv(L.nr, NT) * NT;
+    }
+    if (a.n == 0) continue;
+    k_urow_max<<<a.n / NT, NT, 0, st>>>(a);
+    SSAMG_LAUNCH_CHECK();
+  }
+}
+
+void launch_urb(const std::vector<Level>& lev, cudaStream_t st) {
+  const int nlev = (int)lev.size();
+  for (int l = 0; l < nlev;) {
+    UrbArgs a{};
+    for (; l < nlev && a.nl < SSAMG_DINV_LEVELS; ++l) {
+      const Level& L = lev[l];
+      if (!L.u_rb) continue;
+      a.lv[a.nl++] = UrbLevel{L.u_ptr, L.u_rb, L.nr, a.n, nullptr};
+      a.n += L.nublk;
+    }
+    if (a.n == 0) continue;
+    k_urb<<<cdiv(a.n, NT), NT, 0, st>>>(a);
+    SSAMG_LAUNCH_CHECK();
+  }
+}
 
 void launch_dinv(const std::vector<Level>& lev, int first, int last, int relax, double factor,
                  bool fp32, cudaStream_t st) {

@@ -42,6 +42,10 @@
 #define SSAMG_RP_FILL 0.8    // and the least fraction of their brick cells inside the parts
 #define SSAMG_TPR 4       // fewest lanes per U row in row jobs
 #define SSAMG_TPR_MAX 16  // most lanes per U row (levels whose rows are long)
+#define SSAMG_UROW_ENTRIES 256  // U entries per block of an entry-balanced row job
+#define SSAMG_UROW_CELLS_F32 300000  // largest levels that take them, by the cycle's precision
+#define SSAMG_UROW_CELLS_F64 40000
+#define SSAMG_UROW_SLOTS 2      // entries a thread of it fetches ahead
 
 // ---------------------------------------------------------------------------
 // Division by a run-time constant (round-up multiply-high method of Granlund
@@ -175,7 +179,9 @@ struct LevelView {
   const T* u_rw;        // column cell (centre, -d*, +d*; -1 absent) and the two side weights
   T* uy;                // dense per-cell (U x)(c) of the vector last passed to a row job; 0 off rows
   int nr;
-  int nublk;            // blocks of row jobs (SSAMG_BLOCK / tpr rows each)
+  const int4* u_rb;     // rows of every row-job block: first row, rows, first and end entry
+                        // (null: SSAMG_BLOCK / tpr rows each)
+  int nublk;            // blocks of row jobs
   int tpr;              // lanes per U row in row jobs (4, 8 or 16)
   // inside a PCG solve: the problems' scalars; a block of a problem whose
   // iteration has stopped leaves its cycle work undone (nothing reads it)
@@ -325,6 +331,7 @@ struct Level {
   float* u_rw32 = nullptr;
   double* uy64 = nullptr;
   float* uy32 = nullptr;
+  int4* u_rb = nullptr;
   int nublk = 0;
   int tpr = SSAMG_TPR;
   // cycle work vectors (precision of the cycle)
@@ -341,13 +348,13 @@ template <>
 inline LevelView<double> Level::view<double>() const {
   return LevelView<double>{d_parts, d_blk, d_bblk, d_fblk, d_cellstart, np, (int)N, coef, dinv, Pw, Pe,
                            u_map, u_ptr, u_col, u_val, u_bits, u_rows, u_pj, u_pw, u_rj, u_rw, uy64, nr,
-                           nublk, tpr, g_ssamg_skip, 1, 0, 0};
+                           u_rb, nublk, tpr, g_ssamg_skip, 1, 0, 0};
 }
 template <>
 inline LevelView<float> Level::view<float>() const {
   return LevelView<float>{d_parts, d_blk, d_bblk, d_fblk, d_cellstart, np, (int)N, coef32, dinv32, Pw32,
                           Pe32, u_map, u_ptr, u_col, u_val32, u_bits, u_rows, u_pj, u_pw32, u_rj,
-                          u_rw32, uy32, nr, nublk, tpr, g_ssamg_skip, 1, 0, 0};
+                          u_rw32, uy32, nr, u_rb, nublk, tpr, g_ssamg_skip, 1, 0, 0};
 }
 
 struct SsamgError {
@@ -478,6 +485,10 @@ void launch_relax_final(const Level& L, const T* x, const T* b, double* z, const
                         double* zprev, double* partial, cudaStream_t st);
 // row-job setup data of L's couplings: P rows (L.u_pj set) and restriction
 // rows from the level above Fp (L.u_rj set)
+// longest U row of every level (maxrow[l], zeroed by the caller), and u_rb of
+// every level that has it, one launch per SSAMG_DINV_LEVELS levels
+void launch_urow_max(const std::vector<Level>& lev, int* maxrow, cudaStream_t st);
+void launch_urb(const std::vector<Level>& lev, cudaStream_t st);
 void launch_ucols(const Level* Fp, const Level& L, bool fp32, bool pj, bool rj, cudaStream_t st);
 template <class T>
 void launch_residual(const Level& L, const T* x, const T* b, T* r, cudaStream_t st);
