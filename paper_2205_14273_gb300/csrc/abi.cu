@@ -1023,7 +1023,7 @@ bool valid_tile(int t) {
 // Block starts of a level's launches and the first cell of every part (host
 // side of the level's device tables).
 struct LevelTables {
-  std::vector<int> blk, bblk, fblk, cs;
+  std::vector<int> blk, bblk, fblk, cs, wblk;
 };
 
 // Levels a hierarchy can have: every level halves an extent of some part, and
@@ -1045,7 +1045,8 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
   // tile form: the table's entry for the level's size class, else the
   // built-in rule (SSAMG_CPT_LARGE cells per thread on large levels)
   const int te = s->tiles[tile_class(ntot)];
-  L.cpt = te ? (te & ~SSAMG_TILE_BRICKS) : ntot >= SSAMG_CPT_MIN_CELLS ? SSAMG_CPT_LARGE : 1;
+  L.wcpt = ntot >= SSAMG_CPT_MIN_CELLS ? SSAMG_CPT_LARGE : 1;
+  L.cpt = te ? (te & ~SSAMG_TILE_BRICKS) : L.wcpt;
   L.bricks = te ? (te & SSAMG_TILE_BRICKS) != 0 : 1;
   const long long tile = (long long)L.cpt * SSAMG_BLOCK;
   for (int p = 0; p < np; ++p) {
@@ -1056,6 +1057,10 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
   }
   L.nblk = blk[np];
   L.nfblk = fblk[np];
+  t.wblk.assign(np + 1, 0);
+  for (int p = 0; p < np; ++p)
+    t.wblk[p + 1] = t.wblk[p] + (int)cdivll(L.parts[p].ncell, (long long)L.wcpt * SSAMG_BLOCK);
+  L.nwblk = t.wblk[np];
   // bricks (checked 7-point operator applies)
   std::vector<int>& bblk = t.bblk;
   bblk.assign(np + 1, 0);
@@ -1126,12 +1131,14 @@ void upload_level(ssamg_solver s, Level& L, const Level* next, cudaStream_t st) 
     L.d_bblk = aalloc<int>(s->arena, np + 1);
     L.d_fblk = aalloc<int>(s->arena, np + 1);
     L.d_cellstart = aalloc<int>(s->arena, np + 1);
+    L.d_wblk = aalloc<int>(s->arena, np + 1);
   }
   SSAMG_CUDA(cudaMemcpyAsync(L.d_parts, L.dparts.data(), sizeof(DPart) * np, cudaMemcpyHostToDevice, st));
   SSAMG_CUDA(cudaMemcpyAsync(L.d_blk, t.blk.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
   SSAMG_CUDA(cudaMemcpyAsync(L.d_bblk, t.bblk.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
   SSAMG_CUDA(cudaMemcpyAsync(L.d_fblk, t.fblk.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
   SSAMG_CUDA(cudaMemcpyAsync(L.d_cellstart, t.cs.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
+  SSAMG_CUDA(cudaMemcpyAsync(L.d_wblk, t.wblk.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
 }
 
 // Every level's tables in one device block, through one pinned staging
@@ -1145,7 +1152,7 @@ void upload_levels(ssamg_solver s, cudaStream_t st) {
   for (int l = 0; l < nl; ++l) {
     level_tables(s, s->lev[l], l + 1 < nl ? &s->lev[l + 1] : nullptr, t[l]);
     const size_t np = (size_t)s->lev[l].np;
-    total += al(sizeof(DPart) * np) + 4 * al(sizeof(int) * (np + 1));
+    total += al(sizeof(DPart) * np) + 5 * al(sizeof(int) * (np + 1));
   }
   if (s->h_up_cap < total) {
     pinned_free(s->h_up);
@@ -1170,6 +1177,7 @@ void upload_levels(ssamg_solver s, cudaStream_t st) {
     L.d_bblk = (int*)put(t[l].bblk.data(), sizeof(int) * (np + 1));
     L.d_fblk = (int*)put(t[l].fblk.data(), sizeof(int) * (np + 1));
     L.d_cellstart = (int*)put(t[l].cs.data(), sizeof(int) * (np + 1));
+    L.d_wblk = (int*)put(t[l].wblk.data(), sizeof(int) * (np + 1));
   }
   SSAMG_CUDA(cudaMemcpyAsync(dev, s->h_up, o, cudaMemcpyHostToDevice, st));
 }
@@ -1391,7 +1399,7 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   upload_level(s, L0, nullptr, st);
 
   // ---- Section 3.1: coupling sums c and spacings W (one sync)
-  double* d_partial = aalloc<double>(s->arena, 3ll * L0.nblk);
+  double* d_partial = aalloc<double>(s->arena, 3ll * L0.nwblk);
   double* d_c = aalloc<double>(s->arena, 3ll * np);
   launch_wsum(L0, d_partial, d_c, st);
   s->c.assign(3 * np, 0.0);

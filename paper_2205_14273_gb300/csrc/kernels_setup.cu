@@ -34,11 +34,15 @@ __device__ __forceinline__ int p_row_arrays(const DPart& p, const T* __restrict_
 // the warp's lane 0), multiplied once per block; per-cell entries are summed
 // in FP64 cell by cell.  The diagonal's sign is read from its bits (negative,
 // nonzero, not NaN: the same decision as diag < 0).
-__global__ void __launch_bounds__(NT) k_wsum(LevelView<double> L, double* __restrict__ partial) {
+// The blocks (starts wblk, wcpt cells per thread) are those of the built-in tile
+// rule whatever the level's tile table: a partition that followed the table
+// would round the sums, and with them omega and every cycle, differently.
+__global__ void __launch_bounds__(NT) k_wsum(LevelView<double> L, const int* __restrict__ wblk,
+                                             int wcpt, double* __restrict__ partial) {
   __shared__ DPart sp;
   __shared__ double sh[NT];
   __shared__ int shc[NT / 32][SSAMG_MAXE];
-  int p = block_part(L.blk, L.parts, L.np, sp);
+  const int p = block_part(wblk, L.parts, L.np, sp);
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (lane == 0)
     for (int e = 0; e < SSAMG_MAXE; ++e) shc[w][e] = 0;
@@ -52,9 +56,9 @@ __global__ void __launch_bounds__(NT) k_wsum(LevelView<double> L, double* __rest
       anyvar = true;
   }
   double s0 = 0, s1 = 0, s2 = 0;
-  const int base = ((int)blockIdx.x - sp.blk0) * sp.cpt * SSAMG_BLOCK + (int)threadIdx.x;
+  const int base = ((int)blockIdx.x - wblk[p]) * wcpt * SSAMG_BLOCK + (int)threadIdx.x;
 #pragma unroll 1
-  for (int m = 0; m < sp.cpt; ++m) {
+  for (int m = 0; m < wcpt; ++m) {
     const int c = base + m * SSAMG_BLOCK;
     if (c - lane >= sp.ncell) break;  // the warp's first cell: a warp-uniform exit
     const bool valid = c < sp.ncell;
@@ -1346,8 +1350,11 @@ __global__ void k_mask_part(double* __restrict__ v, int nx, int ny, int nz, int 
 // Launchers
 // ---------------------------------------------------------------------------
 // Block partials of the allocation-free coupling sums: one triple per block
-// of a level launch, every slot written before it is read.
-static __device__ __align__(256) double g_wsum_scratch[3 * SSAMG_NOALLOC_MAX_BLOCKS];
+// of a level launch, every slot written before it is read.  (A tile table of
+// more cells per thread lets a level of up to SSAMG_CPT_MIN_CELLS cells pass
+// the limit with up to that many / SSAMG_BLOCK more blocks of the sums.)
+static __device__ __align__(256) double
+    g_wsum_scratch[3 * (SSAMG_NOALLOC_MAX_BLOCKS + SSAMG_CPT_MIN_CELLS / SSAMG_BLOCK + 1)];
 
 double* wsum_static_scratch() {
   void* p = nullptr;
@@ -1356,9 +1363,9 @@ double* wsum_static_scratch() {
 }
 
 void launch_wsum(const Level& L, double* partial, double* c_out, cudaStream_t st) {
-  k_wsum<<<L.nblk, NT, 0, st>>>(L.view<double>(), partial);
+  k_wsum<<<L.nwblk, NT, 0, st>>>(L.view<double>(), L.d_wblk, L.wcpt, partial);
   SSAMG_LAUNCH_CHECK();
-  k_wfinal<<<L.np, NT, 0, st>>>(L.d_blk, partial, c_out);
+  k_wfinal<<<L.np, NT, 0, st>>>(L.d_wblk, partial, c_out);
   SSAMG_LAUNCH_CHECK();
 }
 

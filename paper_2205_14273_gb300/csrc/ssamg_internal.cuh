@@ -296,7 +296,9 @@ struct Level {
   int* d_bblk = nullptr;
   int* d_fblk = nullptr;
   int* d_cellstart = nullptr;
-  int nblk = 0, nfblk = 0, nbblk = 0;
+  int* d_wblk = nullptr;  // block starts of the coupling sums (the built-in tile rule's)
+  int nblk = 0, nfblk = 0, nbblk = 0, nwblk = 0;
+  int wcpt = 1;
   int cpt = 1;
   int bricks = 1; // 0: the tile table keeps this level's operator applies on cell tiles
   double brick_fill = 0.0;  // cells / (bricks x brick cells): how full the level's bricks are
