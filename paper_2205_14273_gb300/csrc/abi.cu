@@ -352,8 +352,9 @@ struct ssamg_solver_s {
   int tail_blocks = 0;
   int tail_parts = 0;          // part descriptors of the tail levels (single-CTA tail)
   TailBarrier* tail_bar = nullptr;
-  // cluster tail (use_tail = 3): levels ctail.lev[0..nt) from level ctail_lt on
+  // cluster tail (use_tail = 3): ctail_levels levels from level ctail_lt on
   int ctail_lt = -1;
+  int ctail_levels = 0;
   int ctail_nc = 0;
   long long ctail_smem = 0;
   CTailArgs ctail{};
@@ -1235,95 +1236,153 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
   std::vector<int> len(first[Lc + 1] - first[lt]);
   SSAMG_CUDA(cudaMemcpyAsync(len.data(), dlen, sizeof(int) * len.size(), cudaMemcpyDeviceToHost, st));
   SSAMG_CUDA(cudaStreamSynchronize(st));
-  const size_t w = fp32 ? sizeof(float) : sizeof(double);
+  auto level_len = [&](int l) { return len.data() + (first[l] - first[lt]); };
   auto al = [](long long v) { return (v + 15) & ~15ll; };
+  // Lays levels t0 .. t1 out for nc CTAs with elements of w bytes, those from
+  // level tl on local; the last level carries an explicit matrix of its size
+  // when has_inv.  Row pointers of a region lead it (one copy uploads them):
+  // rp[0] bytes of the sliced region, rp[1] of the common one.
+  auto layout = [&](CTailArgs& a, int t0, int t1, int tl, int nc, size_t w, bool has_inv,
+                    long long rp[2]) {
+    a.nt = t1 - t0 + 1;
+    a.jl = std::min(a.nt, tl - t0);
+    a.direct = has_inv;
+    a.nL = (int)s->lev[t1].N;
+    long long vec = 0, reg[2] = {0, 0};
+    for (int j = 0; j < a.nt; ++j) {
+      CTailLevel& v = a.lev[j];
+      v.n = (int)s->lev[t0 + j].N;
+      v.local = t0 + j >= tl;
+      const int slice = (int)cdivll(v.n, nc);
+      v.S = v.local ? v.n : slice;
+      if (v.S >= (1 << SSAMG_CTAIL_LOCAL_BITS)) return false;
+      // lanes per row: as many as leave every row of the slice a group in one
+      // pass (of a local level too, so that its sums keep the cluster's order)
+      // (FP64: few lanes, the pipe takes 16 cycles for each add of a lane tree)
+      v.tpr = 1;
+      while (v.tpr < (w == 8 ? SSAMG_CTAIL_TPR_F64 : 32) && (long long)slice * v.tpr * 2 <= SSAMG_CTAIL_THREADS) v.tpr *= 2;
+      long long& ro = reg[v.local];
+      v.o_rowptr = (int)ro;
+      ro += 4ll * (v.S + 1);
+    }
+    for (int q = 0; q < 2; ++q) rp[q] = reg[q] = al(reg[q]);
+    for (int j = 0; j < a.nt; ++j) {
+      CTailLevel& v = a.lev[j];
+      const int* ln = level_len(t0 + j);
+      long long mx = 0;
+      for (long long g0 = 0; g0 < v.n; g0 += v.S) {
+        long long sum = 0;
+        for (long long g = g0; g < std::min<long long>(v.n, g0 + v.S); ++g) sum += ln[g];
+        mx = std::max(mx, sum);
+      }
+      long long& ro = reg[v.local];
+      v.o_x = (int)vec;  vec += al(v.S * w);
+      v.o_b = (int)vec;  vec += al(v.S * w);
+      v.o_r = (int)vec;  vec += al(v.S * w);
+      v.o_col = (int)ro;    ro += al(2 * mx);
+      v.o_val = (int)ro;    ro += al(w * mx);
+      v.o_dinv = (int)ro;   ro += al(w * v.S);
+      v.o_pcol = v.o_pval = v.o_rcol = v.o_rval = v.o_inv = 0;
+      if (j + 1 < a.nt) {
+        v.o_pcol = (int)ro; ro += al(2ll * 2 * v.S);
+        v.o_pval = (int)ro; ro += al(w * 2 * v.S);
+      }
+      if (j > 0) {
+        v.o_rcol = (int)ro; ro += al(2ll * 3 * v.S);
+        v.o_rval = (int)ro; ro += al(w * 3 * v.S);
+      }
+      if (j + 1 == a.nt && has_inv) {
+        v.o_inv = (int)ro; ro += al(8ll * v.S * a.nL);
+      }
+    }
+    a.o_sb = (int)vec;
+    if (a.dense) vec += al(8ll * a.nL);
+    a.vec_bytes = (int)vec;
+    a.ro_bytes = reg[0];
+    a.lo_bytes = reg[1];
+    return true;
+  };
+  // Row pointers of `a`'s levels into the nc sliced images and the common one.
+  std::vector<std::vector<int>> keep;  // host buffers of copies in flight
+  auto upload_rowptr = [&](const CTailArgs& a, int t0, int nc, const long long rp[2], char* img,
+                           char* common) {
+    keep.emplace_back((size_t)nc * rp[0] / 4, 0);
+    keep.emplace_back((size_t)rp[1] / 4, 0);
+    std::vector<int>& sl = keep[keep.size() - 2];
+    std::vector<int>& co = keep[keep.size() - 1];
+    for (int j = 0; j < a.nt; ++j) {
+      const CTailLevel& v = a.lev[j];
+      const int* ln = level_len(t0 + j);
+      for (int c = 0; c < (v.local ? 1 : nc); ++c) {
+        int* row = v.local ? co.data() + v.o_rowptr / 4 : sl.data() + ((size_t)c * rp[0] + v.o_rowptr) / 4;
+        int acc = 0;
+        for (int li = 0; li < v.S; ++li) {
+          row[li] = acc;
+          const long long g = (long long)c * v.S + li;
+          if (g < v.n) acc += ln[g];
+        }
+        row[v.S] = acc;
+      }
+    }
+    if (rp[0] > 0)
+      SSAMG_CUDA(cudaMemcpy2DAsync(img, (size_t)a.ro_bytes, sl.data(), (size_t)rp[0], (size_t)rp[0], nc,
+                                   cudaMemcpyHostToDevice, st));
+    if (rp[1] > 0)
+      SSAMG_CUDA(cudaMemcpyAsync(common, co.data(), (size_t)rp[1], cudaMemcpyHostToDevice, st));
+  };
+  // images: zeroed, row pointers from the host, the rest by the fill kernel
+  auto images = [&](CTailArgs& a, int t0, int nc, const long long rp[2], bool f32, const double* inv) {
+    const size_t bytes = (size_t)nc * a.ro_bytes + (size_t)a.lo_bytes;
+    char* img = (char*)s->arena.alloc(bytes);
+    char* common = img + (size_t)nc * a.ro_bytes;
+    SSAMG_CUDA(cudaMemsetAsync(img, 0, bytes, st));
+    upload_rowptr(a, t0, nc, rp, img, common);
+    a.image = img;
+    a.common = common;
+    launch_ctail_fill(f32, s->lev, t0, a, inv, img, common, st);
+  };
+  const size_t w = fp32 ? sizeof(float) : sizeof(double);
+  // the first level small enough for the local or dense form, if it is not
+  // the coarsest
+  int small = lt;
+  while (small < Lc && s->lev[small].N > (fp32 ? SSAMG_CTAIL_LOCAL_CELLS : SSAMG_CTAIL_DENSE_CELLS)) ++small;
   for (int nc : {SSAMG_CTAIL_MAX_CTAS, 8}) {
     for (int t0 = lt; t0 < Lc; ++t0) {
-      const int nt = Lc - t0 + 1;
-      if (nt > SSAMG_CTAIL_MAX_LEVELS) continue;
-      CTailArgs a{};
-      a.nt = nt;
-      a.direct = direct;
-      a.nL = (int)s->lev[Lc].N;
-      long long vec = 0, ro = 0;
-      bool ok = true;
-      std::vector<long long> cap(nt);
-      // row pointers of every level first, so that one 2-D copy uploads them
-      for (int j = 0; j < nt; ++j) {
-        a.lev[j].S = (int)cdivll(s->lev[t0 + j].N, nc);
-        a.lev[j].o_rowptr = (int)ro;
-        ro += 4ll * (a.lev[j].S + 1);
+      if (Lc - t0 + 1 > SSAMG_CTAIL_MAX_LEVELS) continue;
+      for (int form = small < Lc ? 1 : 0; form >= 0; --form) {
+        // form 1: levels from max(small, t0) on local (FP32) or dense (FP64)
+        const int tl = std::max(small, t0);
+        if (form && tl >= Lc) continue;
+        const bool dense = form && !fp32;
+        CTailArgs a{};
+        a.dense = dense;
+        long long rp[2];
+        const bool ok = layout(a, t0, dense ? tl : Lc, form && fp32 ? tl : Lc + 1, nc, w,
+                               dense || direct, rp);
+        const long long smem = a.vec_bytes + a.ro_bytes + a.lo_bytes;
+        if (!ok || smem > optin) continue;
+        const bool can = fp32 ? ctail_prepare<float>(nc, smem) : ctail_prepare<double>(nc, smem);
+        if (!can) continue;
+        const double* inv = direct ? s->cinv : nullptr;
+        if (dense) {
+          // the rest of the cycle as a dense matrix
+          CTailArgs c{};
+          long long crp[2];
+          layout(c, tl, Lc, tl, 1, sizeof(double), direct, crp);
+          images(c, tl, 1, crp, false, inv);
+          double* M = aalloc<double>(s->arena, s->lev[tl].N * s->lev[tl].N);
+          launch_ctail_columns(c, M, st);
+          inv = M;
+        }
+        images(a, t0, nc, rp, fp32, inv);
+        SSAMG_CUDA(cudaStreamSynchronize(st));  // `keep` is read by the copies
+        s->ctail = a;
+        s->ctail_lt = t0;
+        s->ctail_levels = Lc - t0 + 1;
+        s->ctail_nc = nc;
+        s->ctail_smem = smem;
+        return;
       }
-      ro = al(ro);
-      const long long rp_bytes = ro;
-      for (int j = 0; j < nt && ok; ++j) {
-        const Level& L = s->lev[t0 + j];
-        CTailLevel& v = a.lev[j];
-        v.n = (int)L.N;
-        v.S = (int)cdivll(L.N, nc);
-        // lanes per row: as many as leave every row of the slice a group in one pass
-        v.tpr = 1;
-        while (v.tpr < 32 && (long long)v.S * v.tpr * 2 <= SSAMG_CTAIL_THREADS) v.tpr *= 2;
-        if (v.S >= (1 << SSAMG_CTAIL_LOCAL_BITS)) ok = false;
-        long long mx = 0;
-        for (int c = 0; c < nc; ++c) {
-          long long sum = 0;
-          for (long long g = (long long)c * v.S; g < std::min<long long>(L.N, (long long)(c + 1) * v.S); ++g)
-            sum += len[first[t0 + j] - first[lt] + g];
-          mx = std::max(mx, sum);
-        }
-        cap[j] = mx;
-        v.o_x = (int)vec;  vec += al(v.S * w);
-        v.o_b = (int)vec;  vec += al(v.S * w);
-        v.o_r = (int)vec;  vec += al(v.S * w);
-        v.o_col = (int)ro;    ro += al(2 * mx);
-        v.o_val = (int)ro;    ro += al(w * mx);
-        v.o_dinv = (int)ro;   ro += al(w * v.S);
-        v.o_pcol = v.o_pval = v.o_rcol = v.o_rval = v.o_inv = 0;
-        if (j + 1 < nt) {
-          v.o_pcol = (int)ro; ro += al(2ll * 2 * v.S);
-          v.o_pval = (int)ro; ro += al(w * 2 * v.S);
-        }
-        if (j > 0) {
-          v.o_rcol = (int)ro; ro += al(2ll * 3 * v.S);
-          v.o_rval = (int)ro; ro += al(w * 3 * v.S);
-        }
-        if (j + 1 == nt && direct) {
-          v.o_inv = (int)ro; ro += al(8ll * v.S * a.nL);
-        }
-      }
-      if (!ok || vec + ro > optin) continue;
-      a.vec_bytes = (int)vec;
-      a.ro_bytes = ro;
-      const bool can = fp32 ? ctail_prepare<float>(nc, vec + ro) : ctail_prepare<double>(nc, vec + ro);
-      if (!can) break;  // try fewer CTAs
-      // images: zeroed, row pointers from the host, the rest by the fill kernels
-      char* img = (char*)s->arena.alloc((size_t)nc * ro);
-      SSAMG_CUDA(cudaMemsetAsync(img, 0, (size_t)nc * ro, st));
-      std::vector<int> rp((size_t)nc * rp_bytes / 4, 0);
-      for (int j = 0; j < nt; ++j) {
-        const CTailLevel& v = a.lev[j];
-        for (int c = 0; c < nc; ++c) {
-          int* row = rp.data() + ((size_t)c * rp_bytes + v.o_rowptr) / 4;
-          int acc = 0;
-          for (int li = 0; li < v.S; ++li) {
-            row[li] = acc;
-            const long long g = (long long)c * v.S + li;
-            if (g < v.n) acc += len[first[t0 + j] - first[lt] + g];
-          }
-          row[v.S] = acc;
-        }
-      }
-      SSAMG_CUDA(cudaMemcpy2DAsync(img, (size_t)ro, rp.data(), (size_t)rp_bytes, (size_t)rp_bytes,
-                                   nc, cudaMemcpyHostToDevice, st));
-      launch_ctail_fill(fp32, s->lev, t0, a, direct ? s->cinv : nullptr, img, ro, st);
-      SSAMG_CUDA(cudaStreamSynchronize(st));  // rp is a host temporary
-      a.image = img;
-      s->ctail = a;
-      s->ctail_lt = t0;
-      s->ctail_nc = nc;
-      s->ctail_smem = vec + ro;
-      return;
     }
   }
 }
@@ -2968,7 +3027,7 @@ extern "C" int ssamg_tail_levels(ssamg_solver s, int* first, int* ctas, long lon
   if (first) *first = on ? s->ctail_lt : -1;
   if (ctas) *ctas = on ? s->ctail_nc : 0;
   if (smem_bytes) *smem_bytes = on ? s->ctail_smem : 0;
-  return on ? s->ctail.nt : 0;
+  return on ? s->ctail_levels : 0;
 }
 
 extern "C" int ssamg_num_levels(ssamg_solver s) {

@@ -17,11 +17,27 @@
 // relaxation (Eq. relax0).  Every row is summed in a fixed order (its
 // entries strided over a group of lanes, then a fixed shuffle tree), so a tail
 // result is the same bit for bit from run to run.
+//
+// The smallest levels (at most SSAMG_CTAIL_LOCAL_CELLS cells) cost the same
+// four barriers and remote round trips as the others, ~3.8 us (FP32) and
+// ~4.7 us (FP64) each, with nothing to spread.  In FP32 every CTA holds them
+// whole and runs them for itself: block barriers and its own shared memory,
+// each row summed as the cluster would.  In FP64 an SM's two multiply-adds per
+// clock forbid that (256 rows x 30 entries are 2 us an apply); there the rest
+// of the cycle from the first such level down, a linear map of its right-hand
+// side, is formed at setup as a dense matrix (one block per column runs that
+// sub-cycle on a unit vector) and applied like the coarsest inverse, one
+// barrier and 65,536 multiply-adds over the cluster.
+// Measured (tail of one cycle): 13 levels of one part, FP64 61.6 -> 26.7 us;
+// 10 levels of 8 parts, FP64 59 -> 37 us, FP32 38.4 -> 26 us; 13 levels of two
+// parts, FP32 43 -> 29 us.  A row's arithmetic is a small part of a step: four
+// barriers of ~0.3-0.5 us and a remote round trip remain per cluster level.
 #include <cooperative_groups.h>
 
 #include <map>
 #include <mutex>
 #include <tuple>
+#include <type_traits>
 
 #include "kernels_common.cuh"
 
@@ -92,6 +108,7 @@ struct CTailFillArgs {
   int nl, nL;
   long long ro_bytes;
   char* image;
+  char* common;
   int b0[SSAMG_CTAIL_MAX_LEVELS + 1];
   CTailFillLevel lev[SSAMG_CTAIL_MAX_LEVELS];
 };
@@ -104,14 +121,14 @@ __device__ __forceinline__ void ctail_fill_row(const LevelView<double>& L,
                                                const double* __restrict__ inv, int nL,
                                                const CTailLevel& lv, int Sm, int Sn,
                                                char* __restrict__ image, long long ro_bytes,
-                                               int g) {
+                                               char* __restrict__ common, int g) {
   // a warp per row: the stencil entries one per lane (slots by ballot, in
   // entry order), the coupling entries strided over the lanes, the rest by
   // lane 0
   const int lane = threadIdx.x & 31;
   if (g >= L.N) return;
   const int owner = g / lv.S, li = g - owner * lv.S;
-  char* img = image + owner * ro_bytes;
+  char* img = lv.local ? common : image + owner * ro_bytes;
   const int* rowptr = reinterpret_cast<const int*>(img + lv.o_rowptr);
   unsigned short* col = reinterpret_cast<unsigned short*>(img + lv.o_col);
   T* val = reinterpret_cast<T*>(img + lv.o_val);
@@ -201,7 +218,7 @@ __global__ void __launch_bounds__(256) k_ctail_fill(const __grid_constant__ CTai
   const CTailFillLevel& v = A.lev[l];
   const int g = ((int)blockIdx.x - A.b0[l]) * 8 + (int)(threadIdx.x >> 5);
   ctail_fill_row<T>(v.L, v.dinv, v.fm, v.has_fm, v.ln, v.has_p, v.inv, A.nL, v.lv, v.Sm, v.Sn,
-                    A.image, A.ro_bytes, g);
+                    A.image, A.ro_bytes, A.common, g);
 }
 
 // Cluster-wide barrier between the tail's steps.  The non-aligned forms of
@@ -217,14 +234,66 @@ __device__ __forceinline__ void ctail_sync() {
 }
 
 // Value of a packed column of vector `off` (byte offset of that level's
-// vector in every CTA's shared memory).
+// vector in every CTA's shared memory); of a local level, from this CTA's own.
 template <class T>
 __device__ __forceinline__ T ctail_get(cg::cluster_group& cl, char* sm, int off,
-                                       unsigned short pk) {
+                                       unsigned short pk, int local = 0) {
+  if (local) return reinterpret_cast<const T*>(sm + off)[pk];
   const unsigned o = pk >> SSAMG_CTAIL_LOCAL_BITS;
   const unsigned l = pk & ((1u << SSAMG_CTAIL_LOCAL_BITS) - 1u);
   const T* base = cl.map_shared_rank(reinterpret_cast<T*>(sm + off), o);
   return base[l];
+}
+
+// The same over all rows of a level, x in this CTA's shared memory: four rows
+// per lane group at a time (their loads and shuffles overlap).
+template <class T, class Epi>
+__device__ __forceinline__ void ctail_apply_local(const T* x, const CTailLevel& L, const int* rp,
+                                                  const unsigned short* col, const T* val,
+                                                  Epi&& epi) {
+  constexpr int U = 4;
+  const int tpr = L.tpr;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rpw = 32 / tpr, stride = (CT / 32) * rpw;
+  const int sub = lane / tpr, k = lane & (tpr - 1);
+  for (int r0 = warp * rpw; r0 < L.S; r0 += U * stride) {
+    int q[U], q1[U];
+    T acc[U];
+    bool more = false;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int li = r0 + u * stride + sub;
+      acc[u] = (T)0;
+      q[u] = li < L.S ? rp[li] + k : 0;
+      q1[u] = li < L.S ? rp[li + 1] : 0;
+      more |= q[u] < q1[u];
+    }
+    while (more) {
+      T v[U], a[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        v[u] = q[u] < q1[u] ? x[col[q[u]]] : (T)0;
+        a[u] = q[u] < q1[u] ? val[q[u]] : (T)0;
+      }
+      more = false;
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        if (q[u] < q1[u]) acc[u] = fma(a[u], v[u], acc[u]);
+        q[u] += tpr;
+        more |= q[u] < q1[u];
+      }
+    }
+    __syncwarp();
+    for (int o = tpr >> 1; o > 0; o >>= 1) {
+#pragma unroll
+      for (int u = 0; u < U; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int li = r0 + u * stride + sub;
+      if (li < L.S && k == 0) epi(li, acc[u]);
+    }
+  }
 }
 
 // Operator apply over the CSR rows of one level's slice: L.tpr lanes take a
@@ -262,6 +331,119 @@ __device__ __forceinline__ void ctail_apply(cg::cluster_group& cl, char* sm, int
   }
 }
 
+// Sum of entries [q, q1) of a local level's row by G neighbouring lanes, lane
+// h of them holding the partial sums of ctail_apply's lanes h, h + G, ... in
+// registers: its tree (a level of at most SSAMG_CTAIL_LOCAL_CELLS cells has 32
+// lanes a row there), within a lane as far as it goes, so the result is the
+// same bit for bit with log2 G shuffles.  All lanes of the warp call.
+template <int G, class T>
+__device__ __forceinline__ T ctail_row_sum(const T* x, const unsigned short* col, const T* val,
+                                           int q, int q1) {
+  constexpr int K = 32 / G;
+  T a[K];
+#pragma unroll
+  for (int j = 0; j < K; ++j) a[j] = q + G * j < q1 ? val[q + G * j] * x[col[q + G * j]] : (T)0;
+  for (q += 32; q < q1; q += 32) {
+#pragma unroll
+    for (int j = 0; j < K; ++j)
+      if (q + G * j < q1) a[j] = fma(val[q + G * j], x[col[q + G * j]], a[j]);
+  }
+#pragma unroll
+  for (int o = K / 2; o > 0; o >>= 1) {
+#pragma unroll
+    for (int j = 0; j < o; ++j) a[j] += a[j + o];
+  }
+#pragma unroll
+  for (int o = G / 2; o > 0; o >>= 1) a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+  return a[0];
+}
+
+// Operator apply over the rows of a local level by all threads of the CTA:
+// as many lanes per row as give every row a group at once, the row's result to
+// epi on its first lane.
+template <class T, class Epi>
+__device__ __forceinline__ void ctail_apply_rows(const CTailLevel& L, const T* x, const char* ro,
+                                                 Epi&& epi) {
+  const int* rp = reinterpret_cast<const int*>(ro + L.o_rowptr);
+  const unsigned short* col = reinterpret_cast<const unsigned short*>(ro + L.o_col);
+  const T* val = reinterpret_cast<const T*>(ro + L.o_val);
+  auto rows = [&](auto g) {
+    constexpr int G = decltype(g)::value;
+    const int li = threadIdx.x / G, h = threadIdx.x % G;
+    if ((int)(threadIdx.x & ~31u) / G >= L.n) return;  // (whole warps)
+    const bool in = li < L.n;
+    const T v = ctail_row_sum<G, T>(x, col, val, in ? rp[li] + h : 0, in ? rp[li + 1] : 0);
+    if (in && h == 0) epi(li, v);
+  };
+  static_assert(SSAMG_CTAIL_LOCAL_CELLS * 2 <= CT, "two lanes for every row");
+  if (L.n > CT / 4)
+    rows(std::integral_constant<int, 2>{});
+  else if (L.n > CT / 8)
+    rows(std::integral_constant<int, 4>{});
+  else
+    rows(std::integral_constant<int, 8>{});
+}
+
+// The local levels jl .. nt - 1 in this CTA (b and x of level jl are in its
+// shared memory): down, the last level and up, ending with the corrected x
+// of level jl.
+template <class T>
+__device__ __forceinline__ void ctail_local_cycle(const CTailArgs& a, int jl, char* sm,
+                                                  const char* ro) {
+  const int li = threadIdx.x, nt = a.nt;
+  auto vec = [&](int off) { return reinterpret_cast<T*>(sm + off); };
+  for (int l = jl; l + 1 < nt; ++l) {
+    const CTailLevel& L = a.lev[l];
+    const CTailLevel& C = a.lev[l + 1];
+    const T* b = vec(L.o_b);
+    T* r = vec(L.o_r);
+    __syncthreads();  // x of level l
+    ctail_apply_rows<T>(L, vec(L.o_x), ro, [&](int i, T ax) { r[i] = b[i] - ax; });
+    __syncthreads();  // r of level l
+    if (li < C.n) {
+      const unsigned short* rc = reinterpret_cast<const unsigned short*>(ro + C.o_rcol);
+      const T* rv = reinterpret_cast<const T*>(ro + C.o_rval);
+      T v = rv[li] * r[rc[li]];
+      v = fma(rv[C.S + li], r[rc[C.S + li]], v);
+      v = fma(rv[2 * C.S + li], r[rc[2 * C.S + li]], v);
+      vec(C.o_b)[li] = v;
+      vec(C.o_x)[li] = reinterpret_cast<const T*>(ro + C.o_dinv)[li] * v;
+    }
+  }
+  if (a.direct) {
+    const CTailLevel& L = a.lev[nt - 1];
+    __syncthreads();  // b of the last level
+    if (li < L.n) {
+      const double* iv = reinterpret_cast<const double*>(ro + L.o_inv) + (long long)li * a.nL;
+      const T* b = vec(L.o_b);
+      double s = 0.0;
+#pragma unroll 8
+      for (int t = 0; t < a.nL; ++t) s = fma(iv[t], (double)b[t], s);
+      vec(L.o_x)[li] = (T)s;
+    }
+  }
+  for (int l = nt - 2; l >= jl; --l) {
+    const CTailLevel& L = a.lev[l];
+    const CTailLevel& C = a.lev[l + 1];
+    const T* e = vec((l + 1 == nt - 1) ? C.o_x : C.o_r);
+    const T* b = vec(L.o_b);
+    T* x = vec(L.o_x);
+    T* out = vec(L.o_r);
+    __syncthreads();  // x of level l+1
+    if (li < L.n) {
+      const unsigned short* pc = reinterpret_cast<const unsigned short*>(ro + L.o_pcol);
+      const T* pv = reinterpret_cast<const T*>(ro + L.o_pval);
+      T v = x[li];
+      v = fma(pv[li], e[pc[li]], v);
+      v = fma(pv[L.S + li], e[pc[L.S + li]], v);
+      x[li] = v;
+    }
+    __syncthreads();  // x + P e of level l
+    const T* dv = reinterpret_cast<const T*>(ro + L.o_dinv);
+    ctail_apply_rows<T>(L, x, ro, [&](int i, T ax) { out[i] = fma(dv[i], b[i] - ax, x[i]); });
+  }
+}
+
 // The tail of one V(1,1) cycle: from the right-hand side of level T (global,
 // b_top) to the corrected x of level T (global, x_top).
 template <class T>
@@ -271,42 +453,54 @@ __global__ void __launch_bounds__(CT, 1) k_ctail(const CTailArgs a, const T* b_t
   cg::cluster_group cl = cg::this_cluster();
   const int c = (int)cl.block_rank();
   const int tid = threadIdx.x;
-  // the read-only image (setup data) first, then the wait for the
+  // the read-only images (setup data) first, then the wait for the
   // predecessor that wrote b_top
   {
     const int4* src = reinterpret_cast<const int4*>(a.image + (long long)c * a.ro_bytes);
     int4* dst = reinterpret_cast<int4*>(sm + a.vec_bytes);
-    const long long n16 = a.ro_bytes / 16;
-    for (long long t = tid; t < n16; t += CT) dst[t] = src[t];
+    const int n16 = (int)(a.ro_bytes / 16);
+#pragma unroll 4
+    for (int t = tid; t < n16; t += CT) dst[t] = src[t];
+    src = reinterpret_cast<const int4*>(a.common);
+    dst += n16;
+    const int l16 = (int)(a.lo_bytes / 16);
+#pragma unroll 4
+    for (int t = tid; t < l16; t += CT) dst[t] = src[t];
   }
   pdl_wait();
   __syncthreads();  // the image (read below: level T's diagonal) is staged
   const int nt = a.nt;
+  const char* const ro_s = sm + a.vec_bytes;
+  const char* const ro_l = ro_s + a.ro_bytes;
+  auto ro_of = [&](const CTailLevel& L) { return L.local ? ro_l : ro_s; };
+  auto apply = [&](const CTailLevel& L, auto&& epi) {
+    ctail_apply<T>(cl, sm, L.o_x, L, reinterpret_cast<const int*>(ro_s + L.o_rowptr),
+                   reinterpret_cast<const unsigned short*>(ro_s + L.o_col),
+                   reinterpret_cast<const T*>(ro_s + L.o_val), epi);
+  };
   {
     const CTailLevel& L = a.lev[0];
     T* b = reinterpret_cast<T*>(sm + L.o_b);
     T* x = reinterpret_cast<T*>(sm + L.o_x);
-    const T* dv = reinterpret_cast<const T*>(sm + a.vec_bytes + L.o_dinv);
+    const T* dv = reinterpret_cast<const T*>(ro_of(L) + L.o_dinv);
     for (int li = tid; li < L.S; li += CT) {
-      const int g = c * L.S + li;
+      const int g = (L.local ? 0 : c * L.S) + li;
       const T v = g < L.n ? b_top[g] : (T)0;
       b[li] = v;
       x[li] = dv[li] * v;  // pre-relaxation from zero
     }
   }
   // down: residual, then restriction with the coarse level's pre-relaxation
-  for (int l = 0; l + 1 < nt; ++l) {
+  // (onto the first local level every CTA restricts all of it)
+  for (int l = 0; l + 1 < nt && !a.lev[l].local; ++l) {
     const CTailLevel& L = a.lev[l];
     const CTailLevel& C = a.lev[l + 1];
-    const char* ro = sm + a.vec_bytes;
-    const int* rp = reinterpret_cast<const int*>(ro + L.o_rowptr);
-    const unsigned short* col = reinterpret_cast<const unsigned short*>(ro + L.o_col);
-    const T* val = reinterpret_cast<const T*>(ro + L.o_val);
     const T* b = reinterpret_cast<const T*>(sm + L.o_b);
     T* r = reinterpret_cast<T*>(sm + L.o_r);
     ctail_sync();  // x of level l complete in every CTA
-    ctail_apply<T>(cl, sm, L.o_x, L, rp, col, val, [&](int li, T ax) { r[li] = b[li] - ax; });
+    apply(L, [&](int li, T ax) { r[li] = b[li] - ax; });
     ctail_sync();  // r of level l complete
+    const char* ro = ro_of(C);
     const unsigned short* rc = reinterpret_cast<const unsigned short*>(ro + C.o_rcol);
     const T* rv = reinterpret_cast<const T*>(ro + C.o_rval);
     const T* dvc = reinterpret_cast<const T*>(ro + C.o_dinv);
@@ -320,13 +514,38 @@ __global__ void __launch_bounds__(CT, 1) k_ctail(const CTailArgs a, const T* b_t
       xc[li] = dvc[li] * v;
     }
   }
-  // coarsest level: the dense inverse (FP64) or one relaxation sweep
-  {
+  if (a.jl < nt) {
+    if constexpr (sizeof(T) == 4)  // (FP64 has no local levels)
+      ctail_local_cycle<T>(a, a.jl, sm, ro_l);
+    __syncthreads();  // the corrected x of the first local level
+  } else if (a.direct) {
+    // last level: its explicit matrix (FP64)
     const CTailLevel& L = a.lev[nt - 1];
     T* x = reinterpret_cast<T*>(sm + L.o_x);
-    if (a.direct) {
-      ctail_sync();  // b of the coarsest level complete
-      const double* iv = reinterpret_cast<const double*>(sm + a.vec_bytes + L.o_inv);
+    const double* iv = reinterpret_cast<const double*>(ro_s + L.o_inv);
+    ctail_sync();  // b of the last level
+    if (a.dense) {
+      // every CTA gathers b, then eight lanes per row of its slice
+      double* sb = reinterpret_cast<double*>(sm + a.o_sb);
+      for (int t = tid; t < a.nL; t += CT) {
+        const int o = t / L.S;
+        sb[t] = (double)cl.map_shared_rank(reinterpret_cast<T*>(sm + L.o_b), o)[t - o * L.S];
+      }
+      __syncthreads();
+      constexpr int DL = 8;  // lanes per row (each add of a lane tree takes the FP64 pipe 16 cycles)
+      for (int l0 = 0; l0 < L.S; l0 += CT / DL) {
+        const int li = l0 + tid / DL;
+        double s = 0.0;
+        if (li < L.S) {
+          const double* row = iv + (long long)li * a.nL;
+#pragma unroll 8
+          for (int t = tid % DL; t < a.nL; t += DL) s = fma(row[t], sb[t], s);
+        }
+        if (l0 + (tid & ~31) / DL < L.S)  // (warps with a row)
+          for (int o = DL / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (li < L.S && tid % DL == 0) x[li] = (T)s;
+      }
+    } else {
       for (int li = tid; li < L.S; li += CT) {
         double s = 0.0;
         if (c * L.S + li < L.n) {
@@ -350,33 +569,29 @@ __global__ void __launch_bounds__(CT, 1) k_ctail(const CTailArgs a, const T* b_t
         x[li] = (T)s;
       }
     }
-    // (without the direct solve x = omega M^-1 b is already there)
   }
+  // (without the direct solve x = omega M^-1 b is already there)
   // up: prolongation x_l += P x_{l+1}, then post-relaxation into r_l
-  for (int l = nt - 2; l >= 0; --l) {
+  for (int l = min(nt - 2, a.jl - 1); l >= 0; --l) {
     const CTailLevel& L = a.lev[l];
     const CTailLevel& C = a.lev[l + 1];
-    const char* ro = sm + a.vec_bytes;
+    const char* ro = ro_s;
     const int xcoff = (l + 1 == nt - 1) ? C.o_x : C.o_r;  // the corrected x of level l+1
     const unsigned short* pc = reinterpret_cast<const unsigned short*>(ro + L.o_pcol);
     const T* pv = reinterpret_cast<const T*>(ro + L.o_pval);
     T* x = reinterpret_cast<T*>(sm + L.o_x);
-    ctail_sync();  // x of level l+1 complete
+    if (!C.local) ctail_sync();  // x of level l+1
     for (int li = tid; li < L.S; li += CT) {
       T v = x[li];
-      v = fma(pv[li], ctail_get<T>(cl, sm, xcoff, pc[li]), v);
-      v = fma(pv[L.S + li], ctail_get<T>(cl, sm, xcoff, pc[L.S + li]), v);
+      v = fma(pv[li], ctail_get<T>(cl, sm, xcoff, pc[li], C.local), v);
+      v = fma(pv[L.S + li], ctail_get<T>(cl, sm, xcoff, pc[L.S + li], C.local), v);
       x[li] = v;
     }
     ctail_sync();  // x + P e of level l complete
-    const int* rp = reinterpret_cast<const int*>(ro + L.o_rowptr);
-    const unsigned short* col = reinterpret_cast<const unsigned short*>(ro + L.o_col);
-    const T* val = reinterpret_cast<const T*>(ro + L.o_val);
     const T* dv = reinterpret_cast<const T*>(ro + L.o_dinv);
     const T* b = reinterpret_cast<const T*>(sm + L.o_b);
     T* out = reinterpret_cast<T*>(sm + L.o_r);
-    ctail_apply<T>(cl, sm, L.o_x, L, rp, col, val,
-                   [&](int li, T ax) { out[li] = fma(dv[li], b[li] - ax, x[li]); });
+    apply(L, [&](int li, T ax) { out[li] = fma(dv[li], b[li] - ax, x[li]); });
   }
   // the corrected x of level T (own slice) to global memory; its rows were
   // written by the first lanes of the row groups
@@ -384,12 +599,91 @@ __global__ void __launch_bounds__(CT, 1) k_ctail(const CTailArgs a, const T* b_t
   {
     const CTailLevel& L = a.lev[0];
     const T* res = reinterpret_cast<const T*>(sm + (nt > 1 ? L.o_r : L.o_x));
-    for (int li = tid; li < L.S; li += CT) {
-      const int g = c * L.S + li;
-      if (g < L.n) x_top[g] = res[li];
-    }
+    if (!L.local || c == 0)
+      for (int li = tid; li < L.S; li += CT) {
+        const int g = (L.local ? 0 : c * L.S) + li;
+        if (g < L.n) x_top[g] = res[li];
+      }
   }
   ctail_sync();  // no CTA leaves while another may still read its shared memory
+}
+
+// Column blockIdx.x of the dense matrix of the levels of `a` (all local, FP64):
+// their cycle applied to the unit vector, vectors in shared memory, the image
+// read where it lies (L1 and L2 hold it).
+__global__ void __launch_bounds__(CT) k_ctail_columns(const CTailArgs a, double* dense) {
+  extern __shared__ __align__(16) char sm[];
+  const int tid = threadIdx.x;
+  const int nt = a.nt;
+  auto vec = [&](int off) { return reinterpret_cast<double*>(sm + off); };
+  auto ro = [&](int off) { return a.common + off; };
+  auto apply = [&](const CTailLevel& L, auto&& epi) {
+    ctail_apply_local<double>(vec(L.o_x), L, reinterpret_cast<const int*>(ro(L.o_rowptr)),
+                              reinterpret_cast<const unsigned short*>(ro(L.o_col)),
+                              reinterpret_cast<const double*>(ro(L.o_val)), epi);
+  };
+  {
+    const CTailLevel& L = a.lev[0];
+    const double* dv = reinterpret_cast<const double*>(ro(L.o_dinv));
+    for (int li = tid; li < L.S; li += CT) {
+      const double v = li == (int)blockIdx.x ? 1.0 : 0.0;
+      vec(L.o_b)[li] = v;
+      vec(L.o_x)[li] = dv[li] * v;
+    }
+  }
+  for (int l = 0; l + 1 < nt; ++l) {
+    const CTailLevel& L = a.lev[l];
+    const CTailLevel& C = a.lev[l + 1];
+    const double* b = vec(L.o_b);
+    double* r = vec(L.o_r);
+    __syncthreads();
+    apply(L, [&](int li, double ax) { r[li] = b[li] - ax; });
+    __syncthreads();
+    const unsigned short* rc = reinterpret_cast<const unsigned short*>(ro(C.o_rcol));
+    const double* rv = reinterpret_cast<const double*>(ro(C.o_rval));
+    const double* dvc = reinterpret_cast<const double*>(ro(C.o_dinv));
+    for (int li = tid; li < C.S; li += CT) {
+      double v = rv[li] * r[rc[li]];
+      v = fma(rv[C.S + li], r[rc[C.S + li]], v);
+      v = fma(rv[2 * C.S + li], r[rc[2 * C.S + li]], v);
+      vec(C.o_b)[li] = v;
+      vec(C.o_x)[li] = dvc[li] * v;
+    }
+  }
+  __syncthreads();
+  if (a.direct) {
+    const CTailLevel& L = a.lev[nt - 1];
+    const double* iv = reinterpret_cast<const double*>(ro(L.o_inv));
+    for (int li = tid; li < L.S; li += CT) {
+      double s = 0.0;
+      for (int t = 0; t < a.nL; ++t) s = fma(iv[li * a.nL + t], vec(L.o_b)[t], s);
+      vec(L.o_x)[li] = s;
+    }
+  }
+  for (int l = nt - 2; l >= 0; --l) {
+    const CTailLevel& L = a.lev[l];
+    const CTailLevel& C = a.lev[l + 1];
+    const double* e = vec((l + 1 == nt - 1) ? C.o_x : C.o_r);
+    const unsigned short* pc = reinterpret_cast<const unsigned short*>(ro(L.o_pcol));
+    const double* pv = reinterpret_cast<const double*>(ro(L.o_pval));
+    double* x = vec(L.o_x);
+    __syncthreads();
+    for (int li = tid; li < L.S; li += CT) {
+      double v = x[li];
+      v = fma(pv[li], e[pc[li]], v);
+      v = fma(pv[L.S + li], e[pc[L.S + li]], v);
+      x[li] = v;
+    }
+    __syncthreads();
+    const double* dv = reinterpret_cast<const double*>(ro(L.o_dinv));
+    const double* b = vec(L.o_b);
+    double* out = vec(L.o_r);
+    apply(L, [&](int li, double ax) { out[li] = fma(dv[li], b[li] - ax, x[li]); });
+  }
+  __syncthreads();
+  const CTailLevel& L = a.lev[0];
+  const double* res = vec(nt > 1 ? L.o_r : L.o_x);
+  for (int li = tid; li < L.S; li += CT) dense[(long long)li * L.n + blockIdx.x] = res[li];
 }
 
 inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -421,13 +715,14 @@ void launch_ctail_rowlen(const std::vector<Level>& lev, int first, int last, int
 }
 
 void launch_ctail_fill(bool fp32, const std::vector<Level>& lev, int t0, const CTailArgs& ta,
-                       const double* inv, char* image, long long ro_bytes, cudaStream_t st) {
+                       const double* inv, char* image, char* common, cudaStream_t st) {
   const int nt = ta.nt;
   CTailFillArgs a{};
   a.nl = nt;
   a.nL = ta.nL;
-  a.ro_bytes = ro_bytes;
+  a.ro_bytes = ta.ro_bytes;
   a.image = image;
+  a.common = common;
   int nb = 0;
   for (int j = 0; j < nt; ++j) {
     const Level& L = lev[t0 + j];
@@ -450,6 +745,11 @@ void launch_ctail_fill(bool fp32, const std::vector<Level>& lev, int t0, const C
     k_ctail_fill<float><<<nb, 256, 0, st>>>(a);
   else
     k_ctail_fill<double><<<nb, 256, 0, st>>>(a);
+  SSAMG_LAUNCH_CHECK();
+}
+
+void launch_ctail_columns(const CTailArgs& a, double* dense, cudaStream_t st) {
+  k_ctail_columns<<<a.lev[0].n, CT, (size_t)a.vec_bytes, st>>>(a, dense);
   SSAMG_LAUNCH_CHECK();
 }
 

@@ -207,29 +207,41 @@ struct LevelView {
 // Coarse-level transition run by one thread-block cluster (kernels_tail.cu):
 // per tail level, the rows are split into slices of S rows, one per CTA; a
 // column index packs the owning CTA (high bits) and the position in its slice
-// (SSAMG_CTAIL_LOCAL_BITS low bits).  Offsets are in bytes: vectors within the
-// CTA's vector region, the rest within its read-only region (its image).
+// (SSAMG_CTAIL_LOCAL_BITS low bits).  Local levels (the last ones) are held
+// whole by every CTA (S = n).  Offsets are in bytes: vectors within the CTA's
+// vector region, the rest within its read-only region (its image), for local
+// levels within the common region (the same in every CTA).
 #define SSAMG_CTAIL_THREADS 512
 #define SSAMG_CTAIL_MAX_LEVELS 32
 #define SSAMG_CTAIL_LOCAL_BITS 12
 #define SSAMG_CTAIL_MAX_CTAS 16
 #define SSAMG_CTAIL_CELLS 4096  // default largest level of the cluster tail
+// Levels of at most this many cells: FP32 local in every CTA, FP64 folded
+// into one dense matrix (see kernels_tail.cu)
+#define SSAMG_CTAIL_LOCAL_CELLS 256
+#define SSAMG_CTAIL_DENSE_CELLS 256
+#define SSAMG_CTAIL_TPR_F64 4  // most lanes per CSR row in FP64
 struct CTailLevel {
   int n, S;                  // cells, rows per CTA slice
+  int local;                 // 1: whole in every CTA
   int tpr;                   // lanes per CSR row in the operator applies (power of two <= 32)
   int o_x, o_b, o_r;         // the level's vectors
   int o_rowptr, o_col, o_val, o_dinv;  // CSR of A = S + U (local row pointers), omega M^-1
   int o_pcol, o_pval;        // P's row of each fine cell (2 per row), to the next level
   int o_rcol, o_rval;        // restriction row of each coarse cell (3 per row), from the level above
-  int o_inv;                 // coarsest level: rows of the explicit inverse (FP64)
+  int o_inv;                 // last level: rows of the explicit inverse or of the dense matrix (FP64)
 };
 struct CTailArgs {
   const char* image;         // NC images of ro_bytes each
-  long long ro_bytes;
+  const char* common;        // the local levels' image, lo_bytes
+  long long ro_bytes, lo_bytes;
   int vec_bytes;
-  int nt;                    // tail levels (>= 2)
-  int direct;                // 1: coarsest level by the explicit inverse, 0: one relaxation sweep
-  int nL;                    // cells of the coarsest level
+  int nt;                    // tail levels in this form (>= 1)
+  int jl;                    // first local level (nt: none)
+  int direct;                // 1: last level by its explicit matrix, 0: one relaxation sweep
+  int dense;                 // 1: that matrix is the rest of the cycle (a warp per row)
+  int o_sb;                  // dense: the last level's b gathered (FP64)
+  int nL;                    // cells of the last level
   CTailLevel lev[SSAMG_CTAIL_MAX_LEVELS];
 };
 
@@ -531,7 +543,10 @@ void launch_coarse_inverse(int n, const double* Lfac, double* inv, cudaStream_t 
 void launch_ctail_rowlen(const std::vector<Level>& lev, int first, int last, int* const* len,
                          cudaStream_t st);
 void launch_ctail_fill(bool fp32, const std::vector<Level>& lev, int t0, const CTailArgs& ta,
-                       const double* inv, char* image, long long ro_bytes, cudaStream_t st);
+                       const double* inv, char* image, char* common, cudaStream_t st);
+// dense (n x n, n = a.lev[0].n): one cycle over the levels of `a` (all local,
+// FP64 common image) applied to every unit vector.
+void launch_ctail_columns(const CTailArgs& a, double* dense, cudaStream_t st);
 // Allows the tail kernel nc-CTA clusters and smem bytes of shared memory per
 // CTA; false when the device cannot run such a cluster.
 template <class T>
