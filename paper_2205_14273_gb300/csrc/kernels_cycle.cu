@@ -1552,20 +1552,10 @@ __global__ void __launch_bounds__(NT) k_exp(int n, const double* gg, double* kap
   if (c < n) kap[c] = exp(gg[c]);
 }
 
-__global__ void __launch_bounds__(NT) k_diffusion_exp_gradient(LevelView<double> L,
-                                                               const double* kap,
-                                                               const double* lam,
-                                                               const double* x,
-                                                               double* dg) {
-  pdl_trigger();
-  pdl_wait();
-  __shared__ DPart sp;
-  stage_part(sp, L.parts);
-  __syncthreads();
-  int c = blockIdx.x * NT + threadIdx.x;
-  if (c >= sp.ncell) return;
-  int i, j, k;
-  cell_coords(sp, c, i, j, k);
+// dL/dg at cell c = (i, j, k) from its six faces, a division each: the form
+// for coefficients beyond the shared-face kernel's range.
+__device__ __forceinline__ double dg_cell(const DPart& sp, const double* kap, const double* lam,
+                                          const double* x, int c, int i, int j, int k) {
   const double kc = kap[c];
   const double lc = lam[c], xc = x[c];
   const int sx = 1, sy = sp.n[0], sz = sp.n[0] * sp.n[1];
@@ -1587,7 +1577,146 @@ __global__ void __launch_bounds__(NT) k_diffusion_exp_gradient(LevelView<double>
   face(j < sp.n[1] - 1, sy);
   face(k > 0, -sz);
   face(k < sp.n[2] - 1, sz);
-  dg[c] = kc * acc;
+  return kc * acc;
+}
+
+// 1 / s for s in [2^-200, 2^200] (else `bad` is set and the value is not
+// used): an approximate FP32 reciprocal of the mantissa, widened by integer
+// operations, and one third-order Newton step y (1 + e + e^2), e = 1 - s y
+// (Newton-Raphson iteration with the quadratic term of the series; e < 2^-21,
+// so the remaining error e^3 is below FP64 rounding).  Three FP64
+// instructions; a division takes about nine.
+__device__ __forceinline__ double rcp_fp64(double s, bool& bad) {
+  const int hi = __double2hiint(s);
+  const int ex = (hi >> 20) - 1023;  // (s < 0, infinity and NaN fall outside the range too)
+  bad |= (unsigned)(ex + 200) > 400u;
+  const float f = __uint_as_float(0x3f800000u | ((unsigned)(hi & 0xfffff) << 3) |
+                                  ((unsigned)__double2loint(s) >> 29));
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+  const unsigned rb = __float_as_uint(r);
+  const double y = __hiloint2double((int)(rb >> 3) + ((896 - ex) << 20), (int)(rb << 29));
+  const double e = fma(-s, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+
+// dL/dg of the exp-diffusion operator.  A face between cells c and n adds
+// -2 k_n^2 t to c's sum and -2 k_c^2 t to n's, t = (lam_c - lam_n)
+// (x_c - x_n) / (k_c + k_n)^2, so each face's t is formed once and handed to
+// both cells.  The kernel is bound by the FP64 pipe (2 multiply-adds per clock
+// and SM on this GPU): with a face per cell and side and a division each it
+// took 102 FP64 instructions a cell, here ~40 (9 per face and its reciprocal
+// without conversions; the exponential before it another 15).  128^3: 455 ->
+// 235 us with the exponential.
+// A block takes a GX x GY column of cells, GZ planes of it: the plane's kappa,
+// kappa^2, lambda and x with a halo in shared memory (double-buffered along
+// z), t of the faces towards +x and +y through shared memory, that towards
+// +z kept in a register for the next plane.  The faces between two blocks are
+// computed by both, packed into two warps (40 beside the block's own 768 a
+// plane).  When a coefficient lies beyond rcp_fp64's range the block takes
+// dg_cell for its cells.
+constexpr int GX = 32, GY = 8, GZ = 8, GP = GX + 2;
+__global__ void __launch_bounds__(NT) k_diffusion_exp_gradient(LevelView<double> L,
+                                                               const double* kap,
+                                                               const double* lam,
+                                                               const double* x,
+                                                               double* dg, int nbx, int nby) {
+  static_assert(GX * GY == NT && GX == 32, "a warp per row");
+  pdl_trigger();
+  __shared__ DPart sp;
+  __shared__ double sk[2][(GY + 2) * GP], sq[2][(GY + 2) * GP], sl[2][(GY + 2) * GP],
+      sx[2][(GY + 2) * GP];
+  __shared__ double tx[GY][GX + 1], ty[GY + 1][GX];
+  stage_part(sp, L.parts);
+  __syncthreads();
+  pdl_wait();
+  const int nx = sp.n[0], ny = sp.n[1], nz = sp.n[2], nxy = nx * ny;
+  const int bx = blockIdx.x % nbx, byz = blockIdx.x / nbx;
+  const int i0 = bx * GX, j0 = (byz % nby) * GY, k0 = (byz / nby) * GZ;
+  const int kend = min(k0 + GZ, nz);
+  const int t = threadIdx.x, ti = t % GX, tj = t / GX;
+  const int i = i0 + ti, j = j0 + tj;
+  const bool in = i < nx && j < ny;
+  const int ctr = (tj + 1) * GP + ti + 1;
+  // the halo cell this thread loads (no corners): rows j0 - 1 and j0 + GY, columns
+  // i0 - 1 and i0 + GX
+  int hpos = -1, hi_ = 0, hj = 0;
+  if (t < 2 * GX) {
+    hi_ = i0 + ti;
+    hj = t < GX ? j0 - 1 : j0 + GY;
+    hpos = (t < GX ? 0 : GY + 1) * GP + ti + 1;
+  } else if (t < 2 * GX + 2 * GY) {
+    const int u = t - 2 * GX;
+    hi_ = u < GY ? i0 - 1 : i0 + GX;
+    hj = j0 + u % GY;
+    hpos = (u % GY + 1) * GP + (u < GY ? 0 : GX + 1);
+  }
+  const bool hin = hpos >= 0 && hi_ >= 0 && hi_ < nx && hj >= 0 && hj < ny;
+  const int c0 = j * nx + i, h0 = hj * nx + hi_;
+  // (cells outside the box: kappa 1, lambda and x 0; their faces are not used)
+  auto put = [&](int buf, int pos, bool ok, int c) {
+    const double kv = ok ? kap[c] : 1.0;
+    sk[buf][pos] = kv;
+    sq[buf][pos] = kv * kv;
+    sl[buf][pos] = ok ? lam[c] : 0.0;
+    sx[buf][pos] = ok ? x[c] : 0.0;
+  };
+  bool bad = false;
+  auto face = [&](bool ok, double ka, double la, double xa, double kb, double lb, double xb) {
+    const double s = ka + kb;
+    bool b = false;
+    const double h = rcp_fp64(s * s, b);
+    bad |= b && ok;
+    const double v = h * ((la - lb) * (xa - xb));
+    return ok ? v : 0.0;
+  };
+  auto face_at = [&](int buf, bool ok, int a, int b) {
+    return face(ok, sk[buf][a], sl[buf][a], sx[buf][a], sk[buf][b], sl[buf][b], sx[buf][b]);
+  };
+  put(0, ctr, in, k0 * nxy + c0);
+  if (hpos >= 0) put(0, hpos, hin, k0 * nxy + h0);
+  // the face towards -z of the first plane
+  double tz = 0.0, qm = 0.0;
+  if (k0 > 0) {
+    const int c = (k0 - 1) * nxy + c0;
+    const double km = in ? kap[c] : 1.0;
+    qm = km * km;
+    tz = face(in, km, in ? lam[c] : 0.0, in ? x[c] : 0.0, sk[0][ctr], sl[0][ctr], sx[0][ctr]);
+  }
+  __syncthreads();
+  int buf = 0;
+  for (int k = k0; k < kend; ++k, buf ^= 1) {
+    const bool up = k + 1 < nz;
+    put(buf ^ 1, ctr, in && up, (k + 1) * nxy + c0);
+    if (hpos >= 0 && k + 1 < kend) put(buf ^ 1, hpos, hin, (k + 1) * nxy + h0);
+    tx[tj][ti + 1] = face_at(buf, in && i + 1 < nx, ctr, ctr + 1);
+    ty[tj + 1][ti] = face_at(buf, in && j + 1 < ny, ctr, ctr + GP);
+    if (t < GX)  // faces towards -y of the block's first row
+      ty[0][ti] = face_at(buf, i < nx && j0 > 0, ti + 1, GP + ti + 1);
+    else if (t < GX + GY)  // and towards -x of its first column
+      tx[ti][0] = face_at(buf, j0 + ti < ny && i0 > 0, (ti + 1) * GP, (ti + 1) * GP + 1);
+    const double tp = face(in && up, sk[buf][ctr], sl[buf][ctr], sx[buf][ctr], sk[buf ^ 1][ctr],
+                           sl[buf ^ 1][ctr], sx[buf ^ 1][ctr]);
+    __syncthreads();
+    if (in) {
+      const double* q = sq[buf];
+      double acc = q[ctr - 1] * tx[tj][ti];
+      acc = fma(q[ctr + 1], tx[tj][ti + 1], acc);
+      acc = fma(q[ctr - GP], ty[tj][ti], acc);
+      acc = fma(q[ctr + GP], ty[tj + 1][ti], acc);
+      acc = fma(qm, tz, acc);
+      acc = fma(sq[buf ^ 1][ctr], tp, acc);
+      acc += acc;
+      const int nb = (i == 0) + (i == nx - 1) + (j == 0) + (j == ny - 1) + (k == 0) + (k == nz - 1);
+      if (nb) acc = fma((double)nb, sl[buf][ctr] * sx[buf][ctr], acc);  // Dirichlet faces
+      dg[k * nxy + c0] = -sk[buf][ctr] * acc;
+    }
+    qm = sq[buf][ctr];
+    tz = tp;
+    __syncthreads();
+  }
+  if (__syncthreads_or(bad) && in)
+    for (int k = k0; k < kend; ++k) dg[k * nxy + c0] = dg_cell(sp, kap, lam, x, k * nxy + c0, i, j, k);
 }
 
 }  // namespace
@@ -2023,7 +2152,9 @@ void launch_diffusion_exp_gradient(const Level& L, const double* g, const double
   const int n = (int)L.parts[0].ncell;
   launch_k(k_exp, cdiv(n, NT), NT, 0, st, n, g, kap);
   SSAMG_LAUNCH_CHECK();
-  launch_k(k_diffusion_exp_gradient, cdiv(n, NT), NT, 0, st, L.view<double>(), (const double*)kap,
-           lam, x, dg);
+  const int* e = L.parts[0].n;
+  const int nbx = cdiv(e[0], GX), nby = cdiv(e[1], GY);
+  launch_k(k_diffusion_exp_gradient, nbx * nby * cdiv(e[2], GZ), NT, 0, st, L.view<double>(),
+           (const double*)kap, lam, x, dg, nbx, nby);
   SSAMG_LAUNCH_CHECK();
 }
