@@ -259,6 +259,25 @@ __device__ __forceinline__ T stencil7_canon_checked(const DPart& p, const T* __r
   return acc;
 }
 
+// The 27 entries in offset-code order, every entry per cell.
+template <class T>
+__device__ __forceinline__ T stencil27_checked(const DPart& p, const T* __restrict__ a,
+                                               const T* __restrict__ xc, int i, int j, int k) {
+  const int nx = p.n[0], nxy = p.n[0] * p.n[1], s = p.ncell;
+  const bool xm = i > 0, xp = i < p.n[0] - 1, ym = j > 0, yp = j < p.n[1] - 1, zm = k > 0,
+             zp = k < p.n[2] - 1;
+  T acc = (T)0;
+#pragma unroll
+  for (int e = 0; e < 27; ++e) {
+    const int dx = e % 3 - 1, dy = (e / 3) % 3 - 1, dz = e / 9 - 1;
+    const bool ok = (dx == 0 || (dx < 0 ? xm : xp)) && (dy == 0 || (dy < 0 ? ym : yp)) &&
+                    (dz == 0 || (dz < 0 ? zm : zp));
+    const T xv = xc[ok ? dx + dy * nx + dz * nxy : 0];
+    acc = fma(a[e * s], ok ? xv : (T)0, acc);
+  }
+  return acc;
+}
+
 template <int K, class T>
 __device__ __forceinline__ T stencil_checked_fixed(const DPart& p, const T* __restrict__ coef,
                                                    const T* __restrict__ xc, int c, int i, int j,
