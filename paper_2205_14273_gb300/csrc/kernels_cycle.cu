@@ -971,6 +971,8 @@ __device__ __forceinline__ T tail_apply(const LevelView<T>& L, const DPart& sp,
     case SH_C27: return apply_A_sh<SH_C27>(L, sp, x, c);
     case SH_UGEN: return apply_A_sh<SH_UGEN>(L, sp, x, c);
     case SH_K7: return apply_A_sh<SH_K7>(L, sp, x, c);
+    case SH_U9: return apply_A_sh<SH_U9>(L, sp, x, c);
+    case SH_K5: return apply_A_sh<SH_K5>(L, sp, x, c);
     default: return apply_A_sh<SH_CHECKED>(L, sp, x, c);
   }
 }
@@ -1202,7 +1204,8 @@ __global__ void k_cast_f2d(const float* in, double* out, int n) {
 // 52.9 -> 39.1 us with the U x launch before it, of 25 us for the FP64 pipe (7
 // multiply-adds a cell).
 template <int K>
-__global__ void __launch_bounds__(NT, 4) k_matvec(LevelView<double> L, const double* x, double* y) {
+__global__ void __launch_bounds__(NT, K == 15 ? 2 : K == 27 ? 3 : 4)
+    k_matvec(LevelView<double> L, const double* x, double* y) {
   pdl_trigger();
   __shared__ DPart sp;
   block_part(L.blk, L.parts, L.np, sp);
@@ -1830,6 +1833,8 @@ void launch_relax0_u(const Level& L, const T* b, T* x, cudaStream_t st) {
     case SH_C27: { constexpr int SHV = SH_C27; KCALL; } break; \
     case SH_UGEN: { constexpr int SHV = SH_UGEN; KCALL; } break; \
     case SH_K7: { constexpr int SHV = SH_K7; KCALL; } break;   \
+    case SH_U9: { constexpr int SHV = SH_U9; KCALL; } break;   \
+    case SH_K5: { constexpr int SHV = SH_K5; KCALL; } break;   \
     default: { constexpr int SHV = SH_CHECKED; KCALL; } break; \
   }
 
@@ -1912,6 +1917,7 @@ void launch_cycle_rhs(const Level& L, int R, long long vstride, int skip_stride,
       T* og = out + o;
       switch (L.shape) {
         case SH_U7: RHS_GROUP_LAUNCH(SH_U7); break;
+        case SH_U9: RHS_GROUP_LAUNCH(SH_U9); break;
         case SH_U15: RHS_GROUP_LAUNCH(SH_U15); break;
         case SH_C27: RHS_GROUP_LAUNCH(SH_C27); break;
         default: RHS_GROUP_LAUNCH(SH_UGEN); break;
