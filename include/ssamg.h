@@ -399,9 +399,9 @@ int ssamg_time_kernel(ssamg_solver s, int kernel, int level, int reps, double* u
  *     and PCG operator applies run over 32 x 8 x 8 bricks, each thread
  *     marching a column along z; the other kernels keep the cell tiles.
  * The tile table has one entry per size class c = floor(log2(max(n, 1))),
- * c = 0 .. SSAMG_TILE_CLASSES - 1: 0 selects the built-in rule (4 cells per
- * thread from 300,000 cells up, 1 below; bricks where the level allows
- * them), k alone selects k cells per thread without bricks, and
+ * c = 0 .. SSAMG_TILE_CLASSES - 1: 0 selects the built-in rule (1 cell per
+ * thread below 300,000 cells, 2 below 622,592, else 4; bricks where the
+ * level allows them), k alone selects k cells per thread without bricks, and
  * k | SSAMG_TILE_BRICKS k cells per thread with bricks allowed.  A tile form
  * decides only which thread computes which cell: every cycle result is the
  * same bit for bit under any table; the PCG's dot products, summed per
@@ -417,7 +417,9 @@ int ssamg_set_tile_table(ssamg_solver s, const int* table);
 /* Copies the solver's tile table into table[SSAMG_TILE_CLASSES].  Host only. */
 int ssamg_get_tile_table(ssamg_solver s, int* table);
 /* The tile form level `level` of the set-up hierarchy runs with: cells per
- * thread, and 1 in *bricks when its operator applies run over bricks.
+ * thread, and 1 in *bricks when its operator applies may run over bricks (with
+ * a table entry of SSAMG_TILE_BRICKS they do; under the built-in rule where the
+ * level has enough of them, well filled).
  * Host only. */
 int ssamg_level_tile(ssamg_solver s, int level, int* cells_per_thread, int* bricks);
 /* Tile autotuner: a grid search over the forms {1, 2, 4} cells per thread,

@@ -1047,8 +1047,9 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
   // built-in rule (SSAMG_CPT_LARGE cells per thread on large levels)
   const int te = s->tiles[tile_class(ntot)];
   L.wcpt = ntot >= SSAMG_CPT_MIN_CELLS ? SSAMG_CPT_LARGE : 1;
-  L.cpt = te ? (te & ~SSAMG_TILE_BRICKS) : L.wcpt;
-  L.bricks = te ? (te & SSAMG_TILE_BRICKS) != 0 : 1;
+  L.cpt = te ? (te & ~SSAMG_TILE_BRICKS)
+             : ntot >= SSAMG_CPT_MIN_CELLS && ntot < SSAMG_CPT_WAVE_CELLS ? 2 : L.wcpt;
+  L.bricks = te ? (te & SSAMG_TILE_BRICKS ? 2 : 0) : 1;
   const long long tile = (long long)L.cpt * SSAMG_BLOCK;
   for (int p = 0; p < np; ++p) {
     const PartH& h = L.parts[p];
@@ -2096,7 +2097,7 @@ void enqueue_pcg_body(ssamg_solver s, cudaGraphConditionalHandle h, int use_h, c
   SkipScope skip(s->sc);
   const int npart = vcycle(s, s->r, s->z, st, s->partial, zp);
   if (npart > 0)  // the last relaxation writes partials per block of its tiles
-    launch_pcg_beta_from_partials(L0, s->z, s->p, c, final_ranges(L0, c), st);
+    launch_pcg_beta_from_partials(L0, s->z, s->p, c, final_ranges(L0, c, s->prm.precision == 1), st);
   else
     launch_pcg_beta(L0, s->r, s->z, zp, s->p, c, st);
   launch_pcg_alpha(L0, s->p, s->q, c, st);
@@ -2452,7 +2453,7 @@ int enqueue_vcycle_rhs(ssamg_solver s, bool dots, cudaStream_t st) {
           launch_relax0_u<T>(Ls[0], b0(), (T*)Ls[0].x, st);
         }
       });
-    if (!uses_bricks(Ls[l])) {
+    if (!uses_bricks<T>(Ls[l])) {
       use_rhs(s, 0);
       launch_residual_rhs<T>(Ls[l], R, M.stride[l], s->nprob, (const T*)Ls[l].x,
                              l == 0 ? b0() : (const T*)Ls[l].b, (T*)Ls[l].r, st);
@@ -2487,7 +2488,7 @@ int enqueue_vcycle_rhs(ssamg_solver s, bool dots, cudaStream_t st) {
       });
       return dots ? Ls[0].nblk : 0;
     }
-    if (!uses_bricks(Ls[l])) {
+    if (!uses_bricks<T>(Ls[l])) {
       use_rhs(s, 0);
       T* out = l == 0 ? (T*)s->z : (T*)Ls[l].t;
       launch_relax_rhs<T>(Ls[l], R, M.stride[l], s->nprob, (const T*)Ls[l].r,
@@ -2535,7 +2536,7 @@ void enqueue_pcg_body_rhs(ssamg_solver s, cudaGraphConditionalHandle h, cudaStre
     const PcgCtx c = pcg_ctx(s);
     double* zp = s->prm.flexible ? s->zprev : nullptr;
     if (npart > 0)
-      launch_pcg_beta_from_partials(L0, s->z, s->p, c, final_ranges(L0, c), st);
+      launch_pcg_beta_from_partials(L0, s->z, s->p, c, final_ranges(L0, c, s->prm.precision == 1), st);
     else
       launch_pcg_beta(L0, s->r, s->z, zp, s->p, c, st);
     launch_pcg_alpha(L0, s->p, s->q, c, st);
@@ -3208,7 +3209,7 @@ double time_kernel_us(ssamg_solver s, int kernel, int level, int reps, cudaStrea
         break;
       case 8:  // the PCG's vector steps: beta, p = z + beta p, alpha, x and r updates
         launch_pcg_beta_from_partials(s->lev[0], s->z, s->p, pcg_ctx(s),
-                                      final_ranges(s->lev[0], pcg_ctx(s)), cs);
+                                      final_ranges(s->lev[0], pcg_ctx(s), s->prm.precision == 1), cs);
         launch_pcg_update(s->lev[0], s->p, s->q, s->x, s->r, pcg_ctx(s), 0, 0, cs);
         break;
       case 10: {  // the coarse-level transition's cluster kernel (levels from ctail_lt on)
@@ -3224,7 +3225,8 @@ double time_kernel_us(ssamg_solver s, int kernel, int level, int reps, cudaStrea
       case 11:    // residual of every right-hand side of the last batch solve, one launch
       case 12: {  // relaxation likewise (cell-tile levels above the tail)
         const RhsSet& M = s->rhs;
-        if (M.R < 2 || level >= M.nlev || uses_bricks(L))
+        if (M.R < 2 || level >= M.nlev ||
+            (s->prm.precision == 1 ? uses_bricks<float>(L) : uses_bricks<double>(L)))
           throw SsamgError{SSAMG_ERR_STATE, "no right-hand sides solved together on this level"};
         const RhsSaved saved = save_rhs(s);
         SkipScope none(nullptr);
@@ -3318,7 +3320,7 @@ extern "C" int ssamg_level_tile(ssamg_solver s, int level, int* cells_per_thread
   if (level < 0 || level >= (int)s->lev.size()) return SSAMG_ERR_ARG;
   PdlScope pdl(s->prm);
   *cells_per_thread = s->lev[level].cpt;
-  *bricks = uses_bricks(s->lev[level]) ? 1 : 0;
+  *bricks = brick_level(s->lev[level]) ? 1 : 0;
   return SSAMG_OK;
 }
 
@@ -3388,7 +3390,7 @@ extern "C" int ssamg_autotune(ssamg_solver s, int reps, void* stream, int* table
     prime_pcg(s, st);
     for (int l = 0; l < nl; ++l) {
       // a brick form on a level that cannot use bricks is its cell form
-      if (k >= 0 && (cand[k] & B) && !uses_bricks(s->lev[l])) continue;
+      if (k >= 0 && (cand[k] & B) && !brick_level(s->lev[l])) continue;
       const double t = level_tile_cost(s, l, reps, st);
       if (k < 0) def[l] = t;
       else cost[(size_t)l * nc + k] = t;

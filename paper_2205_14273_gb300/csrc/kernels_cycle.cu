@@ -1789,14 +1789,41 @@ bool rp_bricks(const Level& L) {
          L.brick_fill >= SSAMG_RP_FILL;
 }
 
-bool uses_bricks(const Level& L) {
+bool brick_level(const Level& L) {
   return g_ssamg_bricks && L.bricks && L.shape == SH_K7 && L.nbblk > 0;
 }
 
-// Level-0 block ranges of the problems for the partials that L's operator
-// apply launches write (brick or cell-tile blocks).
-const int* partial_ranges(const Level& L, const PcgCtx& c) { return uses_bricks(L) ? c.pbb : c.pb; }
-const int* final_ranges(const Level& L, const PcgCtx& c) { return uses_bricks(L) ? c.pbb : c.pb; }
+// Whether the operator applies of precision T run over bricks: where the tile
+// table says so, else by the rule.  A brick is one block marching 2048 cells,
+// so a level needs enough of them, well filled; below that the cell tiles
+// spread it further.  Measured (bricks / tiles, us):
+//   FP64 residual, PCG apply, last relaxation: 32^3 (16 bricks) 5.7, 7.8, 9.2 /
+//     2.7, 5.0, 4.6; 8 x 48^3 (576, 0.75 full) 25, 27, 30 / 16, 26, 26; 100^3
+//     (676, 0.72) 22, 29, 44 / 17, 20, 26; 8 x 56^3 (784, 0.88) 30, 37, 43 / 27, 37,
+//     42; 8 x 72^3 (1944, 0.75) 67, 73, 92 / 55, 64, 78; 2 x 96^3 (864, full) 37, 44,
+//     58 / 35, 47, 51; 8 x 64^3 (1024, full) 37, 42, 52 / 37, 48, 60
+//   FP32 residual, last relaxation: 32^3 3.0, 5.8 / 1.5, 3.3; 8 x 33^3 (400, 0.35)
+//     6.6, 12.6 / 3.9, 7.8; 80^3 (300, 0.83) 4.0, 11.7 / 4.2, 7.3; 8 x 48^3 7.6, 13.0
+//     / 6.8, 13.3; 100^3 5.9, 12.9 / 6.7, 12.7; 8 x 64^3 9.9, 24.5 / 14.2, 35.6
+template <class T>
+bool uses_bricks(const Level& L) {
+  if (!brick_level(L)) return false;
+  if (L.bricks == 2) return true;
+  return sizeof(T) == 8 ? L.nbblk >= SSAMG_K7_BRICKS_F64 && L.brick_fill >= SSAMG_K7_FILL_F64
+                        : L.nbblk >= SSAMG_K7_BRICKS_F32 && L.brick_fill >= SSAMG_K7_FILL_F32;
+}
+template bool uses_bricks<float>(const Level&);
+template bool uses_bricks<double>(const Level&);
+
+// Level-0 block ranges of the problems for the partials that L's FP64 operator
+// apply launches write (brick or cell-tile blocks), and the cycle's last
+// relaxation in its precision.
+const int* partial_ranges(const Level& L, const PcgCtx& c) {
+  return uses_bricks<double>(L) ? c.pbb : c.pb;
+}
+const int* final_ranges(const Level& L, const PcgCtx& c, bool fp32) {
+  return (fp32 ? uses_bricks<float>(L) : uses_bricks<double>(L)) ? c.pbb : c.pb;
+}
 
 // Blocks of a launch with nt tile blocks that come before its row jobs.  The
 // entry-balanced row jobs (levels of long rows) go first: their chain of
@@ -1851,7 +1878,7 @@ void launch_relax_final(const Level& L, const T* x, const T* b, double* z, const
   // zprev may be null (no flexible CG): pass a valid buffer and a flag
   const int flex = zprev != nullptr;
   double* zp = flex ? zprev : z;
-  if (uses_bricks(L))
+  if (uses_bricks<T>(L))
     launch_k(pick_km(L.kvar, k7b_relax_final<T, 0>, k7b_relax_final<T, 1>, k7b_relax_final<T, 2>),
              L.nbblk, NT, 0, st, L.view<T>(), x, b, z, rpcg, zp, flex, partial);
   else
@@ -1879,7 +1906,7 @@ void launch_uy(const Level& L, const T* x, cudaStream_t st) {
 
 template <class T>
 void launch_residual(const Level& L, const T* x, const T* b, T* r, cudaStream_t st) {
-  if (uses_bricks(L))
+  if (uses_bricks<T>(L))
     launch_k(pick_km(L.kvar, k7b_residual<T, 0>, k7b_residual<T, 1>, k7b_residual<T, 2>), L.nbblk, NT, 0,
              st, L.view<T>(), x, b, r);
   else
@@ -1888,7 +1915,7 @@ void launch_residual(const Level& L, const T* x, const T* b, T* r, cudaStream_t 
 }
 template <class T>
 void launch_relax(const Level& L, const T* x, const T* b, T* xo, cudaStream_t st) {
-  if (uses_bricks(L))
+  if (uses_bricks<T>(L))
     launch_k(pick_km(L.kvar, k7b_relax<T, 0>, k7b_relax<T, 1>, k7b_relax<T, 2>), L.nbblk, NT, 0,
              st, L.view<T>(), x, b, xo);
   else
@@ -2098,7 +2125,7 @@ void launch_cast_f2d(const float* in, double* out, long long n, cudaStream_t st)
 }
 void launch_matvec(const Level& L, const double* x, double* y, cudaStream_t st) {
   launch_uy<double>(L, x, st);
-  if (uses_bricks(L)) {
+  if (uses_bricks<double>(L)) {
     launch_k(pick_km(L.kvar, k7b_matvec<0>, k7b_matvec<1>, k7b_matvec<2>), L.nbblk, NT, 0, st,
              L.view<double>(), x, y);
   } else {
@@ -2119,7 +2146,7 @@ void launch_matvec(const Level& L, const double* x, double* y, cudaStream_t st) 
 void launch_pcg_init(const Level& L, const double* b, const double* x, double* r,
                      const PcgCtx& c, cudaStream_t st) {
   launch_uy<double>(L, x, st);
-  if (uses_bricks(L))
+  if (uses_bricks<double>(L))
     launch_k(pick_km(L.kvar, k7b_pcg_init<0>, k7b_pcg_init<1>, k7b_pcg_init<2>), L.nbblk, NT, 0,
              st, L.view<double>(), b, x, r, c.partial);
   else
@@ -2160,7 +2187,7 @@ void launch_pcg_beta_from_partials(const Level& L0, const double* z, double* p, 
 void launch_pcg_alpha(const Level& L, const double* p, double* q, const PcgCtx& c,
                       cudaStream_t st) {
   launch_uy<double>(L, p, st);
-  if (uses_bricks(L))
+  if (uses_bricks<double>(L))
     launch_k(pick_km(L.kvar, k7b_spmv_dot<0>, k7b_spmv_dot<1>, k7b_spmv_dot<2>), L.nbblk, NT, 0,
              st, L.view<double>(), p, q, c.partial);
   else
@@ -2184,7 +2211,7 @@ void launch_pcg_update(const Level& L0, const double* p, const double* q, double
 void launch_true_residual(const Level& L, const double* b, const double* x, double* r,
                           const PcgCtx& c, double* out, cudaStream_t st) {
   launch_uy<double>(L, x, st);
-  if (uses_bricks(L))
+  if (uses_bricks<double>(L))
     launch_k(pick_km(L.kvar, k7b_pcg_init<0>, k7b_pcg_init<1>, k7b_pcg_init<2>), L.nbblk, NT, 0,
              st, L.view<double>(), b, x, r, c.partial);
   else

@@ -30,6 +30,12 @@
 #define SSAMG_MAX_PART_BOXES 16  // boxes of one part (ssamg_grid_add_box)
 #define SSAMG_CPT_LARGE 4         // cells per thread on large levels
 #define SSAMG_CPT_MIN_CELLS 300000  // levels smaller than this use one cell per thread
+// Below this many cells blocks of SSAMG_CPT_LARGE cells per thread do not fill
+// one wave (152 SMs x 4 blocks x 1024 cells): two cells per thread, twice the
+// blocks (V-cycles with a level of 442,368 / 521,217 / 524,288 cells: FP32 270 ->
+// 263, FP64 2-D 221 -> 212, FP64 563 -> 551 us; a level of a million cells gains
+// nothing)
+#define SSAMG_CPT_WAVE_CELLS 622592
 #define SSAMG_TUNE_MARGIN 0.97    // a tuned tile form must save 3% of a level's time
 #define SSAMG_TUNE_ITER_MARGIN 0.99  // and the tuned table 1% of a whole PCG iteration
 #define SSAMG_EW 4                 // cells per thread of the elementwise pre-relaxation
@@ -38,6 +44,12 @@
 #define SSAMG_BRICK_X 32
 #define SSAMG_BRICK_Y 8
 #define SSAMG_BRICK_Z 8
+// Fewest bricks of a level, and the least fraction of their cells inside the
+// parts, for the operator applies over bricks (see uses_bricks)
+#define SSAMG_K7_BRICKS_F32 250
+#define SSAMG_K7_FILL_F32 0.6
+#define SSAMG_K7_BRICKS_F64 800
+#define SSAMG_K7_FILL_F64 0.85
 #define SSAMG_RP_BRICKS 152  // fewest bricks for the restriction / prolongation brick forms
 #define SSAMG_RP_FILL 0.8    // and the least fraction of their brick cells inside the parts
 #define SSAMG_TPR 4       // fewest lanes per U row in row jobs
@@ -312,7 +324,7 @@ struct Level {
   int nblk = 0, nfblk = 0, nbblk = 0, nwblk = 0;
   int wcpt = 1;
   int cpt = 1;
-  int bricks = 1; // 0: the tile table keeps this level's operator applies on cell tiles
+  int bricks = 1; // operator applies over bricks: 0 never, 1 by the rule, 2 the table wants them
   double brick_fill = 0.0;  // cells / (bricks x brick cells): how full the level's bricks are
   int kvar = 2;   // per-cell stencil entries: 0 none, 1 only diagonals, 2 others too
   int shape = 0;  // StencilShape of the level's operator apply
@@ -571,13 +583,15 @@ void launch_pcg_beta(const Level& L0, const double* r, const double* z, double* 
                      const PcgCtx& c, cudaStream_t st);
 void launch_pcg_beta_from_partials(const Level& L0, const double* z, double* p, const PcgCtx& c,
                                    const int* ranges, cudaStream_t st);
-// Whether L's operator applies run over bricks, and the per-problem ranges of
-// the partials those launches write.
+// Whether L's operator applies may run over bricks, whether those of precision
+// T do, and the per-problem ranges of the partials their launches write.
+bool brick_level(const Level& L);
+template <class T>
 bool uses_bricks(const Level& L);
 bool rp_bricks(const Level& L);
 const int* partial_ranges(const Level& L, const PcgCtx& c);
 // block ranges of the dot partials the cycle's last relaxation writes
-const int* final_ranges(const Level& L, const PcgCtx& c);
+const int* final_ranges(const Level& L, const PcgCtx& c, bool fp32);
 void launch_pcg_alpha(const Level& L, const double* p, double* q, const PcgCtx& c,
                       cudaStream_t st);
 void launch_pcg_update(const Level& L0, const double* p, const double* q, double* x, double* r,
