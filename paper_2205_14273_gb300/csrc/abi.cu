@@ -1262,9 +1262,12 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
       if (v.S >= (1 << SSAMG_CTAIL_LOCAL_BITS)) return false;
       // lanes per row: as many as leave every row of the slice a group in one
       // pass (of a local level too, so that its sums keep the cluster's order)
-      // (FP64: few lanes, the pipe takes 16 cycles for each add of a lane tree)
+      // (FP64: few lanes, the pipe takes 16 cycles for each add of a lane tree;
+      // the dense matrix's columns have half a block each)
+      const int most = w == 8 ? SSAMG_CTAIL_TPR_F64 : 32;
+      const int threads = nc > 1 ? SSAMG_CTAIL_THREADS : SSAMG_CTAIL_THREADS / 2;
       v.tpr = 1;
-      while (v.tpr < (w == 8 ? SSAMG_CTAIL_TPR_F64 : 32) && (long long)slice * v.tpr * 2 <= SSAMG_CTAIL_THREADS) v.tpr *= 2;
+      while (v.tpr < most && (long long)slice * v.tpr * 2 <= threads) v.tpr *= 2;
       long long& ro = reg[v.local];
       v.o_rowptr = (int)ro;
       ro += 4ll * (v.S + 1);

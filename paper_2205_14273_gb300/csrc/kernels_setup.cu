@@ -57,6 +57,38 @@ __global__ void __launch_bounds__(NT) k_wsum(LevelView<double> L, const int* __r
   }
   double s0 = 0, s1 = 0, s2 = 0;
   const int base = ((int)blockIdx.x - wblk[p]) * wcpt * SSAMG_BLOCK + (int)threadIdx.x;
+  if (sp.canon27 && sp.allvar && sp.zeroext) {
+    // 27 entries per cell, zero outside the box: one sum per set of directions
+    // an entry moves along, combined at the end, an add per entry instead of up
+    // to three (16.8M cells: 2635 -> 940 us; pipe ~760, HBM ~530)
+    double g[8] = {};
+#pragma unroll 1
+    for (int m = 0; m < wcpt; ++m) {
+      const int c = base + m * SSAMG_BLOCK;
+      if (c >= sp.ncell) break;
+      const double* a = L.coef + sp.coef[0] + c;
+      const long long bits = __double_as_longlong(a[13ll * sp.ncell]);
+      const long long mag = bits & 0x7fffffffffffffffll;
+      const bool neg = bits < 0 && mag != 0 && mag <= 0x7ff0000000000000ll;
+      // (the sign through the bits: a select of v or -v becomes two predicated adds)
+      const int flip = neg ? 0 : (int)0x80000000u;
+#pragma unroll
+      for (int z = 0; z < 3; ++z) {
+        double v[9];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) v[e] = a[(long long)(9 * z + e) * sp.ncell];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+          const int set = (e % 3 != 1) | (e / 3 != 1) << 1 | (z != 1) << 2;
+          if (set)
+            g[set] += __hiloint2double(__double2hiint(v[e]) ^ flip, __double2loint(v[e]));
+        }
+      }
+    }
+    s0 = (g[1] + g[3]) + (g[5] + g[7]);
+    s1 = (g[2] + g[3]) + (g[6] + g[7]);
+    s2 = (g[4] + g[5]) + (g[6] + g[7]);
+  } else
 #pragma unroll 1
   for (int m = 0; m < wcpt; ++m) {
     const int c = base + m * SSAMG_BLOCK;
@@ -134,12 +166,67 @@ __global__ void __launch_bounds__(NT) k_wfinal(const int* __restrict__ blk,
 // K2: two-point interpolation weights per fine point (Eq. prolEx, sign
 // reading P = -(plane sum)/(centre-plane sum)), with the part-boundary fix.
 // ---------------------------------------------------------------------------
+// The level's time is the FP64 pipe's: a fine point takes an add per entry and
+// one reciprocal.  The entries are therefore sorted by their offset along d*
+// once per block (a block has one part), so that each is added to its one sum
+// without a test per entry and sum, whose predicated adds had kept the pipe busy
+// three times over; where every entry is per cell and zero outside the box
+// (every coarse level) no entry is tested against the box.  The sums run in
+// entry order as before.  27 entries, 8.4M fine points: 1351 -> 718 us (pipe
+// ~570, HBM ~530).
+template <int K, bool ALLVAR>
+__device__ __forceinline__ void plane_sums(const DPart& sp, const double* __restrict__ coef,
+                                           const signed char (*ord)[9], const int* cnt, int de,
+                                           int c, int i, int j, int k, double* sum, double& diag) {
+  double av[3][K];
+#pragma unroll
+  for (int t = 0; t < 3; ++t)
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      av[t][q] = 0.0;
+      if (q < cnt[t]) {
+        const int e = ord[t][q];
+        if (ALLVAR)
+          av[t][q] = coef[sp.coef[0] + (long long)e * sp.ncell + c];
+        else if (inside(sp, i + sp.o[e][0], j + sp.o[e][1], k + sp.o[e][2]))
+          av[t][q] = coef_at(sp, coef, e, c);
+      }
+    }
+#pragma unroll
+  for (int t = 0; t < 3; ++t) {
+    double v = 0.0;
+#pragma unroll
+    for (int q = 0; q < K; ++q)
+      if (q < cnt[t]) {
+        v += av[t][q];
+        if (t == 1 && ord[1][q] == de) diag = av[1][q];
+      }
+    sum[t] = v;
+  }
+}
+
 __global__ void __launch_bounds__(NT) k_interp(LevelView<double> L, double* __restrict__ Pw,
                                                double* __restrict__ Pe, float* __restrict__ Pw32,
                                                float* __restrict__ Pe32) {
   __shared__ DPart sp;
-  int p = block_part(L.fblk, L.parts, L.np, sp);
+  __shared__ signed char ord[3][9];  // entries by offset along d* (-1, 0, 1), ascending
+  __shared__ int cnt[3];
+  block_part(L.fblk, L.parts, L.np, sp);
   __syncthreads();
+  if (threadIdx.x < 32) {
+    const int e = threadIdx.x;
+    const int od = e < sp.nent ? sp.o[e][sp.dstar] + 1 : -1;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+      const unsigned m = __ballot_sync(0xffffffffu, od == t);
+      if (od == t) ord[t][__popc(m & ((1u << e) - 1u))] = (signed char)e;
+      if (e == 0) cnt[t] = __popc(m);
+    }
+  }
+  __syncthreads();
+  const int most = max(cnt[0], max(cnt[1], cnt[2]));
+  const bool allvar = sp.allvar && sp.zeroext;
+  const int de = sp.slot[13];  // the diagonal entry
   TILE_LOOP_FINE(F, sp) {
     const int d = sp.dstar;
     int fc[3];
@@ -152,32 +239,18 @@ __global__ void __launch_bounds__(NT) k_interp(LevelView<double> L, double* __re
     fc[d] = 2 * fc[d] + 1 - sp.par;  // the fine cell
     const int i = fc[0], j = fc[1], k = fc[2];
     const int c = (k * sp.n[1] + j) * sp.n[0] + i;
-    double nw = 0, ne = 0, den = 0, diag = 0;
-    // entries in batches of IB with predicated loads (in flight together),
-    // summed in entry order as before
-    constexpr int IB = 9;
-    for (int e0 = 0; e0 < sp.nent; e0 += IB) {
-      double av[IB];
-#pragma unroll
-      for (int q = 0; q < IB; ++q) {
-        const int e = e0 + q;
-        const bool ok =
-            e < sp.nent && inside(sp, i + sp.o[e][0], j + sp.o[e][1], k + sp.o[e][2]);
-        av[q] = ok ? coef_at(sp, L.coef, e, c) : 0.0;
-      }
-#pragma unroll
-      for (int q = 0; q < IB; ++q) {
-        const int e = e0 + q;
-        if (e >= sp.nent) break;
-        if (!inside(sp, i + sp.o[e][0], j + sp.o[e][1], k + sp.o[e][2])) continue;
-        const double a = av[q];
-        const int od = sp.o[e][d];
-        if (od < 0) nw += a;
-        else if (od > 0) ne += a;
-        else den += a;
-        if (sp.o[e][0] == 0 && sp.o[e][1] == 0 && sp.o[e][2] == 0) diag += a;
-      }
-    }
+    double sum[3], diag = 0.0;
+    if (!allvar && most <= 5)
+      plane_sums<5, false>(sp, L.coef, ord, cnt, de, c, i, j, k, sum, diag);
+    else if (!allvar)
+      plane_sums<9, false>(sp, L.coef, ord, cnt, de, c, i, j, k, sum, diag);
+    else if (most <= 3)
+      plane_sums<3, true>(sp, L.coef, ord, cnt, de, c, i, j, k, sum, diag);
+    else if (most <= 5)
+      plane_sums<5, true>(sp, L.coef, ord, cnt, de, c, i, j, k, sum, diag);
+    else
+      plane_sums<9, true>(sp, L.coef, ord, cnt, de, c, i, j, k, sum, diag);
+    const double nw = sum[0], den = sum[1], ne = sum[2];
     double pw = 0, pe = 0;
     bool ok = fabs(den) > 1e-300 && ((den > 0) == (diag > 0)) && diag != 0.0;
     if (ok) {
@@ -214,8 +287,11 @@ __global__ void __launch_bounds__(NT) k_interp(LevelView<double> L, double* __re
 // (F its anchor 2I along d*): the product w_a s_o(f) goes to c = t/2 when
 // t = a + o_d is even (g = f + o is a coarse point) and to (t-1)/2 and
 // (t+1)/2 with PW(g), PE(g) when t is odd.  a and o_d are compile-time, so
-// the group's three sums stay in registers; each sum runs in the order
-// (a, o_d) ascending.  Each fine coefficient is read once per coarse cell.
+// the group's three sums stay in registers; the two products that end at the
+// same odd point g are added before they are spread over its P row, which
+// leaves 10 FP64 instructions a group where one product at a time took 19 (the
+// pipe bounds the kernel).  Each fine coefficient is read once per coarse
+// cell.  27 entries, 16.8M -> 8.4M cells: 2726 -> 1747 us (pipe ~1300, HBM ~950).
 // Block b takes group b % 9 of coarse tile b / 9.
 // ---------------------------------------------------------------------------
 // D: the coarsening direction of the part (-1: not coarsened, P = I), a
@@ -267,33 +343,34 @@ __device__ __forceinline__ void rap_group_tile(const LevelView<double>& F, const
       const int nfs[3] = {1, fp.nf[0], fp.nf[0] * fp.nf[1]};
       const int fp_off = fp.poff + q[d1] * nfs[d1] + q[d2] * nfs[d2];
       const int fpi0 = fp.poff + I[d1] * nfs[d1] + I[d2] * nfs[d2];
+      // fine points F - 1, F, F + 1 of this column (w) and of the offset one (G)
+      const bool in[3] = {anchor > 0, true, anchor + 1 < fp.n[dd]};
+      double w[3] = {0.0, 1.0, 0.0}, gw[3] = {0.0, 0.0, 0.0}, ge[3] = {0.0, 0.0, 0.0};
 #pragma unroll
-      for (int a = -1; a <= 1; ++a) {
-        const int fd = anchor + a;
-        if ((unsigned)fd >= (unsigned)fp.n[dd]) continue;
-        const int fcell = cell0 + a * fstr[dd];
-        double w1 = 1.0;
-        if (a != 0) {
-          const int Fi = fpi0 + ((fd + fp.par) >> 1) * nfs[dd];
-          w1 = (a < 0) ? F.Pe[Fi] : F.Pw[Fi];
+      for (int a = 0; a < 3; a += 2)
+        if (in[a]) {
+          const int h = ((anchor + a - 1 + fp.par) >> 1) * nfs[dd];
+          w[a] = a == 0 ? F.Pe[fpi0 + h] : F.Pw[fpi0 + h];
+          gw[a] = F.Pw[fp_off + h];
+          ge[a] = F.Pe[fp_off + h];
         }
-        if (w1 == 0.0) continue;
+      double v[3][3];  // entries o_d = -1, 0, 1 at the three points, zero where absent
 #pragma unroll
-        for (int od = -1; od <= 1; ++od) {
-          const int e = fe[od + 1];
-          const int gd = fd + od;
-          if (e < 0 || (unsigned)gd >= (unsigned)fp.n[dd]) continue;
-          const double v = w1 * coef_at(fp, F.coef, e, fcell);
-          const int t = a + od;
-          if ((t & 1) == 0) {
-            acc[t / 2 + 1] += v;
-          } else {
-            const int Gi = fp_off + ((gd + fp.par) >> 1) * nfs[dd];
-            acc[(t - 1) / 2 + 1] += v * F.Pw[Gi];
-            acc[(t + 1) / 2 + 1] += v * F.Pe[Gi];
-          }
+      for (int a = 0; a < 3; ++a)
+#pragma unroll
+        for (int od = 0; od < 3; ++od) {
+          const int e = fe[od];
+          v[a][od] = e >= 0 && in[a] && (unsigned)(anchor + a + od - 2) < (unsigned)fp.n[dd]
+                         ? coef_at(fp, F.coef, e, cell0 + (a - 1) * fstr[dd])
+                         : 0.0;
         }
-      }
+      const double qm = fma(w[0], v[0][1], v[1][0]);  // at G = F - 1
+      const double qp = fma(w[2], v[2][1], v[1][2]);  // at G = F + 1
+      acc[0] = fma(qm, gw[0], w[0] * v[0][0]);
+      acc[1] = fma(w[0], v[0][2], fma(w[2], v[2][0], v[1][1]));
+      acc[1] = fma(qm, ge[0], acc[1]);
+      acc[1] = fma(qp, gw[2], acc[1]);
+      acc[2] = fma(qp, ge[2], w[2] * v[2][2]);
     }
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
@@ -1015,9 +1092,8 @@ __global__ void __launch_bounds__(NT) k_dinv(const __grid_constant__ DinvArgs A)
     cell_coords(sp, c, i, j, k);
     double v;
     if (A.relax == 0) {
-      double diag = 0.0;
-      for (int e = 0; e < sp.nent; ++e)
-        if (sp.o[e][0] == 0 && sp.o[e][1] == 0 && sp.o[e][2] == 0) diag += coef_at(sp, L.coef, e, c);
+      const int de = sp.slot[13];  // the diagonal entry
+      const double diag = de >= 0 ? coef_at(sp, L.coef, de, c) : 0.0;
       double w = A.factor > 0.0 ? A.factor : sp.omega;
       v = w / diag;
     } else {

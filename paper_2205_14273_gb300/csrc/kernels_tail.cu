@@ -245,54 +245,38 @@ __device__ __forceinline__ T ctail_get(cg::cluster_group& cl, char* sm, int off,
   return base[l];
 }
 
-// The same over all rows of a level, x in this CTA's shared memory: four rows
-// per lane group at a time (their loads and shuffles overlap).
-template <class T, class Epi>
-__device__ __forceinline__ void ctail_apply_local(const T* x, const CTailLevel& L, const int* rp,
-                                                  const unsigned short* col, const T* val,
-                                                  Epi&& epi) {
-  constexpr int U = 4;
+// The same over all rows of a level by NTH threads (tid among them), x in this
+// CTA's shared memory.  For FP64: four entries at a time and then one by one, as
+// an add that is predicated off takes the pipe as long as one that is not.
+template <int NTH, class T, class Epi>
+__device__ __forceinline__ void ctail_apply_local(int tid, const T* x, const CTailLevel& L,
+                                                  const int* rp, const unsigned short* col,
+                                                  const T* val, Epi&& epi) {
   const int tpr = L.tpr;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rpw = 32 / tpr, stride = (CT / 32) * rpw;
+  const int lane = tid & 31, warp = tid >> 5;
+  const int rpw = 32 / tpr;
   const int sub = lane / tpr, k = lane & (tpr - 1);
-  for (int r0 = warp * rpw; r0 < L.S; r0 += U * stride) {
-    int q[U], q1[U];
-    T acc[U];
-    bool more = false;
+  for (int r0 = warp * rpw; r0 < L.S; r0 += (NTH / 32) * rpw) {
+    const int li = r0 + sub;
+    T acc = (T)0;
+    if (li < L.S) {
+      int q = rp[li] + k;
+      const int q1 = rp[li + 1];
+      for (; q + 3 * tpr < q1; q += 4 * tpr) {
+        T v[4], a[4];
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int li = r0 + u * stride + sub;
-      acc[u] = (T)0;
-      q[u] = li < L.S ? rp[li] + k : 0;
-      q1[u] = li < L.S ? rp[li + 1] : 0;
-      more |= q[u] < q1[u];
-    }
-    while (more) {
-      T v[U], a[U];
+        for (int u = 0; u < 4; ++u) {
+          a[u] = val[q + u * tpr];
+          v[u] = x[col[q + u * tpr]];
+        }
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        v[u] = q[u] < q1[u] ? x[col[q[u]]] : (T)0;
-        a[u] = q[u] < q1[u] ? val[q[u]] : (T)0;
+        for (int u = 0; u < 4; ++u) acc = fma(a[u], v[u], acc);
       }
-      more = false;
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (q[u] < q1[u]) acc[u] = fma(a[u], v[u], acc[u]);
-        q[u] += tpr;
-        more |= q[u] < q1[u];
-      }
+      for (; q < q1; q += tpr) acc = fma(val[q], x[col[q]], acc);
     }
     __syncwarp();
-    for (int o = tpr >> 1; o > 0; o >>= 1) {
-#pragma unroll
-      for (int u = 0; u < U; ++u) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int li = r0 + u * stride + sub;
-      if (li < L.S && k == 0) epi(li, acc[u]);
-    }
+    for (int o = tpr >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (li < L.S && k == 0) epi(li, acc);
   }
 }
 
@@ -608,25 +592,41 @@ __global__ void __launch_bounds__(CT, 1) k_ctail(const CTailArgs a, const T* b_t
   ctail_sync();  // no CTA leaves while another may still read its shared memory
 }
 
-// Column blockIdx.x of the dense matrix of the levels of `a` (all local, FP64):
-// their cycle applied to the unit vector, vectors in shared memory, the image
-// read where it lies (L1 and L2 hold it).
-__global__ void __launch_bounds__(CT) k_ctail_columns(const CTailArgs a, double* dense) {
-  extern __shared__ __align__(16) char sm[];
-  const int tid = threadIdx.x;
+// CTAIL_COLS columns of the dense matrix of the levels of `a` (all local, FP64):
+// their cycle applied to unit vectors, a group of CT / CTAIL_COLS threads each,
+// vectors in shared memory, and the image too where it fits (`staged`: read
+// where it lies, every step is two dependent L2 round trips; 256 cells of one
+// part: 94 -> 36 us).
+constexpr int CTAIL_COLS = 2;
+__global__ void __launch_bounds__(CT) k_ctail_columns(const CTailArgs a, int staged, double* dense) {
+  constexpr int NTH = CT / CTAIL_COLS;
+  extern __shared__ __align__(16) char smem[];
+  const int grp = threadIdx.x / NTH, tid = threadIdx.x % NTH;
+  char* const sm = smem + grp * a.vec_bytes;
+  const char* img = a.common;
+  if (staged) {
+    char* to = smem + CTAIL_COLS * a.vec_bytes;
+    const int4* src = reinterpret_cast<const int4*>(a.common);
+    const int n16 = (int)(a.lo_bytes / 16);
+#pragma unroll 8
+    for (int t = threadIdx.x; t < n16; t += CT) reinterpret_cast<int4*>(to)[t] = src[t];
+    img = to;
+    __syncthreads();
+  }
+  const int column = blockIdx.x * CTAIL_COLS + grp;  // (beyond the last: a zero vector, not stored)
   const int nt = a.nt;
   auto vec = [&](int off) { return reinterpret_cast<double*>(sm + off); };
-  auto ro = [&](int off) { return a.common + off; };
+  auto ro = [&](int off) { return img + off; };
   auto apply = [&](const CTailLevel& L, auto&& epi) {
-    ctail_apply_local<double>(vec(L.o_x), L, reinterpret_cast<const int*>(ro(L.o_rowptr)),
+    ctail_apply_local<NTH, double>(tid, vec(L.o_x), L, reinterpret_cast<const int*>(ro(L.o_rowptr)),
                               reinterpret_cast<const unsigned short*>(ro(L.o_col)),
                               reinterpret_cast<const double*>(ro(L.o_val)), epi);
   };
   {
     const CTailLevel& L = a.lev[0];
     const double* dv = reinterpret_cast<const double*>(ro(L.o_dinv));
-    for (int li = tid; li < L.S; li += CT) {
-      const double v = li == (int)blockIdx.x ? 1.0 : 0.0;
+    for (int li = tid; li < L.S; li += NTH) {
+      const double v = li == column ? 1.0 : 0.0;
       vec(L.o_b)[li] = v;
       vec(L.o_x)[li] = dv[li] * v;
     }
@@ -642,7 +642,7 @@ __global__ void __launch_bounds__(CT) k_ctail_columns(const CTailArgs a, double*
     const unsigned short* rc = reinterpret_cast<const unsigned short*>(ro(C.o_rcol));
     const double* rv = reinterpret_cast<const double*>(ro(C.o_rval));
     const double* dvc = reinterpret_cast<const double*>(ro(C.o_dinv));
-    for (int li = tid; li < C.S; li += CT) {
+    for (int li = tid; li < C.S; li += NTH) {
       double v = rv[li] * r[rc[li]];
       v = fma(rv[C.S + li], r[rc[C.S + li]], v);
       v = fma(rv[2 * C.S + li], r[rc[2 * C.S + li]], v);
@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(CT) k_ctail_columns(const CTailArgs a, double*
   if (a.direct) {
     const CTailLevel& L = a.lev[nt - 1];
     const double* iv = reinterpret_cast<const double*>(ro(L.o_inv));
-    for (int li = tid; li < L.S; li += CT) {
+    for (int li = tid; li < L.S; li += NTH) {
       double s = 0.0;
       for (int t = 0; t < a.nL; ++t) s = fma(iv[li * a.nL + t], vec(L.o_b)[t], s);
       vec(L.o_x)[li] = s;
@@ -668,7 +668,7 @@ __global__ void __launch_bounds__(CT) k_ctail_columns(const CTailArgs a, double*
     const double* pv = reinterpret_cast<const double*>(ro(L.o_pval));
     double* x = vec(L.o_x);
     __syncthreads();
-    for (int li = tid; li < L.S; li += CT) {
+    for (int li = tid; li < L.S; li += NTH) {
       double v = x[li];
       v = fma(pv[li], e[pc[li]], v);
       v = fma(pv[L.S + li], e[pc[L.S + li]], v);
@@ -683,7 +683,8 @@ __global__ void __launch_bounds__(CT) k_ctail_columns(const CTailArgs a, double*
   __syncthreads();
   const CTailLevel& L = a.lev[0];
   const double* res = vec(nt > 1 ? L.o_r : L.o_x);
-  for (int li = tid; li < L.S; li += CT) dense[(long long)li * L.n + blockIdx.x] = res[li];
+  if (column < L.n)
+    for (int li = tid; li < L.S; li += NTH) dense[(long long)li * L.n + column] = res[li];
 }
 
 inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -749,7 +750,13 @@ void launch_ctail_fill(bool fp32, const std::vector<Level>& lev, int t0, const C
 }
 
 void launch_ctail_columns(const CTailArgs& a, double* dense, cudaStream_t st) {
-  k_ctail_columns<<<a.lev[0].n, CT, (size_t)a.vec_bytes, st>>>(a, dense);
+  const long long vec = (long long)CTAIL_COLS * a.vec_bytes, all = vec + a.lo_bytes;
+  const int staged = all <= SSAMG_CTAIL_STAGE_BYTES;
+  if (staged)
+    SSAMG_CUDA(cudaFuncSetAttribute(k_ctail_columns, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    SSAMG_CTAIL_STAGE_BYTES));
+  k_ctail_columns<<<cdiv(a.lev[0].n, CTAIL_COLS), CT, (size_t)(staged ? all : vec), st>>>(a, staged,
+                                                                                        dense);
   SSAMG_LAUNCH_CHECK();
 }
 

@@ -232,6 +232,7 @@ struct LevelView {
 // into one dense matrix (see kernels_tail.cu)
 #define SSAMG_CTAIL_LOCAL_CELLS 256
 #define SSAMG_CTAIL_DENSE_CELLS 256
+#define SSAMG_CTAIL_STAGE_BYTES (200 * 1024)  // shared memory of the dense matrix's column blocks
 #define SSAMG_CTAIL_TPR_F64 4  // most lanes per CSR row in FP64
 struct CTailLevel {
   int n, S;                  // cells, rows per CTA slice
