@@ -292,22 +292,24 @@ struct ssamg_matrix_s {
   }
 };
 
+// The instantiated solve graphs, each with the state its launches were captured
+// from (every pointer, count and form they take, see graph_signature): a
+// set-up that leaves all of it as it was (a new operator of the same shape on
+// the same solver walks the same arena) keeps the graph, whose capture and
+// instantiation take 0.2 ms (45 nodes) to 1 ms (four right-hand sides).
 struct GraphSet {
   cudaGraphExec_t pcg = nullptr;
   cudaGraphExec_t vcycle = nullptr;
   cudaGraphExec_t rounds = nullptr;  // several right-hand sides in one graph
-  const double* rounds_b = nullptr;   // the user vectors baked into `rounds`
-  double* rounds_x = nullptr;
-  int rounds_n = 0;
-  int rounds_zero = 1;                // 1: x0 = 0 baked in, 0: x0 read from x
+  std::vector<char> pcg_sig, rounds_sig;
+  static void drop(cudaGraphExec_t& g) {
+    if (g) cudaGraphExecDestroy(g);
+    g = nullptr;
+  }
   void reset() {
-    if (pcg) cudaGraphExecDestroy(pcg);
-    if (vcycle) cudaGraphExecDestroy(vcycle);
-    if (rounds) cudaGraphExecDestroy(rounds);
-    pcg = vcycle = rounds = nullptr;
-    rounds_b = nullptr;
-    rounds_x = nullptr;
-    rounds_n = 0;
+    drop(pcg);
+    drop(vcycle);
+    drop(rounds);
   }
 };
 
@@ -340,6 +342,7 @@ struct ssamg_solver_s {
   Arena arena;
   std::vector<Level> lev;
   ssamg_matrix A = nullptr;
+  std::vector<char> sig;  // graph_signature of the last set-up
   bool ready = false;
   int ndim = 3;
   std::vector<double> c, W;  // nparts x 3
@@ -1402,7 +1405,6 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   const bool fp32 = s->prm.precision == 1;
   s->ndim = ndim;
   s->arena.reset();
-  s->graphs.reset();
   s->rhs = RhsSet{};
   s->lev.clear();
   s->lev.reserve((size_t)s->prm.max_levels + 1);
@@ -2107,6 +2109,70 @@ void enqueue_pcg_body(ssamg_solver s, cudaGraphConditionalHandle h, int use_h, c
   launch_pcg_update(L0, s->p, s->q, s->x, s->r, c, h, use_h, st);
 }
 
+// Everything the captured launches of a solve take from the solver: per level
+// the views and launch forms, the tail, and the PCG's buffers.
+std::vector<char> graph_signature(ssamg_solver s) {
+  std::vector<char> sig;
+  auto put = [&](auto... v) {
+    auto one = [&](auto x) {
+      static_assert(std::is_scalar<decltype(x)>::value, "scalars and pointers only");
+      const char* c = reinterpret_cast<const char*>(&x);
+      sig.insert(sig.end(), c, c + sizeof(x));
+    };
+    (one(v), ...);
+  };
+  sig.reserve(512 * (s->lev.size() + 8));
+  for (const Level& L : s->lev) {
+    put(L.d_parts, L.d_blk, L.d_bblk, L.d_fblk, L.d_cellstart, L.np, L.N, L.coef, L.coef32, L.dinv,
+        L.dinv32, L.Pw, L.Pe, L.Pw32, L.Pe32, L.u_map, L.u_ptr, L.u_rows, L.u_col, L.u_val,
+        L.u_val32, L.u_bits, L.u_pj, L.u_pw, L.u_pw32, L.u_rj, L.u_rw, L.u_rw32, L.uy64, L.uy32);
+    put(L.nr, L.nnz, L.u_rb, L.nublk, L.tpr, L.nblk, L.nfblk, L.nbblk, L.cpt, L.bricks, L.brick_fill,
+        L.kvar, L.shape, L.guard, L.x, L.b, L.r, L.t);
+  }
+  put(s->nprob, s->nL, s->chol, s->cinv, s->tail_lt, s->tail_dev, s->tail_blocks, s->tail_bar,
+      s->tail_parts, s->ctail_lt);
+  if (s->ctail_lt >= 1) {
+    const CTailArgs& a = s->ctail;
+    put(s->ctail_nc, s->ctail_smem, a.image, a.common, a.ro_bytes, a.lo_bytes, a.vec_bytes, a.nt,
+        a.jl, a.direct, a.dense, a.o_sb, a.nL);
+    for (int j = 0; j < a.nt; ++j) {
+      const CTailLevel& v = a.lev[j];
+      put(v.n, v.S, v.local, v.tpr, v.o_x, v.o_b, v.o_r, v.o_rowptr, v.o_col, v.o_val, v.o_dinv,
+          v.o_pcol, v.o_pval, v.o_rcol, v.o_rval, v.o_inv);
+    }
+  }
+  put(s->b, s->x, s->r, s->z, s->p, s->q, s->zprev, s->partial, s->tres, s->sc, s->sc_init, s->ctl,
+      s->hist, s->pb, s->pbb);
+  return sig;
+}
+
+// The same for a graph of nrhs right-hand sides from b to x, its slices when
+// they are solved together.
+std::vector<char> rounds_signature(ssamg_solver s, const double* b, double* x, int nrhs,
+                                   int zero_guess, bool together) {
+  std::vector<char> sig = graph_signature(s);
+  auto put = [&](const void* v, size_t n) {
+    const char* c = static_cast<const char*>(v);
+    sig.insert(sig.end(), c, c + n);
+  };
+  const void* ptr[] = {b, x, s->sc_hist, s->tres_hist};
+  const int num[] = {nrhs, zero_guess, together};
+  put(ptr, sizeof ptr);
+  put(num, sizeof num);
+  if (together) {
+    const RhsSet& M = s->rhs;
+    const void* q[] = {M.pb, M.px, M.pr, M.pz, M.pp, M.pq, M.pzprev, M.partial, M.sc, M.hist};
+    const long long v[] = {M.R, M.nlev, M.stride0, M.partial_len, M.hist_len};
+    put(q, sizeof q);
+    put(v, sizeof v);
+    put(M.stride.data(), M.stride.size() * sizeof(long long));
+    for (const auto* w : {&M.x, &M.b, &M.r, &M.t}) put(w->data(), w->size() * sizeof(char*));
+    put(M.uy32.data(), M.uy32.size() * sizeof(float*));
+    put(M.uy64.data(), M.uy64.size() * sizeof(double*));
+  }
+  return sig;
+}
+
 void build_pcg_graph(ssamg_solver s) {
   if (!s->cs) SSAMG_CUDA(cudaStreamCreateWithFlags(&s->cs, cudaStreamNonBlocking));
   cudaGraph_t g;
@@ -2242,14 +2308,8 @@ void build_rounds_graph(ssamg_solver s, const double* b, double* x, int nrhs, in
                                cudaMemcpyDeviceToDevice, s->cs));
     deps = end();
   }
-  if (s->graphs.rounds) cudaGraphExecDestroy(s->graphs.rounds);
-  s->graphs.rounds = nullptr;
   SSAMG_CUDA(cudaGraphInstantiate(&s->graphs.rounds, g, 0));
   cudaGraphDestroy(g);
-  s->graphs.rounds_b = b;
-  s->graphs.rounds_x = x;
-  s->graphs.rounds_n = nrhs;
-  s->graphs.rounds_zero = zero_guess;
 }
 
 // ---- Right-hand sides solved together --------------------------------------
@@ -2618,8 +2678,6 @@ void build_rhs_graph(ssamg_solver s, const double* b, double* x, int nrhs, int z
     SSAMG_CUDA(cudaMemcpyAsync(saved.sc, s->sc, sizeof(PcgScalars) * np,
                                cudaMemcpyDeviceToDevice, s->cs));
     SSAMG_CUDA(cudaStreamEndCapture(s->cs, &tmp));
-    if (s->graphs.rounds) cudaGraphExecDestroy(s->graphs.rounds);
-    s->graphs.rounds = nullptr;
     SSAMG_CUDA(cudaGraphInstantiate(&s->graphs.rounds, g, 0));
   } catch (...) {
     // leave the capture stream usable: end a capture the error interrupted
@@ -2637,10 +2695,6 @@ void build_rhs_graph(ssamg_solver s, const double* b, double* x, int nrhs, int z
   restore_rhs(s, saved);
   s->any_sc = nullptr;
   cudaGraphDestroy(g);
-  s->graphs.rounds_b = b;
-  s->graphs.rounds_x = x;
-  s->graphs.rounds_n = nrhs;
-  s->graphs.rounds_zero = zero_guess;
 }
 
 // Solves for nrhs right-hand sides (b, x: nrhs x N, device) in one graph
@@ -2657,17 +2711,17 @@ int run_rounds(ssamg_solver s, const double* b, double* x, int nrhs, cudaStream_
     SSAMG_CUDA(cudaMalloc(&s->sc_hist, sizeof(PcgScalars) * np * nrhs));
     SSAMG_CUDA(cudaMalloc(&s->tres_hist, sizeof(double) * 2 * np * nrhs));
     s->hist_cap = nrhs;
-    if (s->graphs.rounds) cudaGraphExecDestroy(s->graphs.rounds);
-    s->graphs.rounds = nullptr;
   }
-  if (!s->graphs.rounds || s->graphs.rounds_b != b || s->graphs.rounds_x != x ||
-      s->graphs.rounds_n != nrhs || s->graphs.rounds_zero != zero_guess) {
-    if (nrhs > 1 && s->prm.rhs_together && rhs_together_ok(s)) {
-      alloc_rhs(s, nrhs, st);
+  const bool together = nrhs > 1 && s->prm.rhs_together && rhs_together_ok(s);
+  if (together) alloc_rhs(s, nrhs, st);
+  std::vector<char> sig = rounds_signature(s, b, x, nrhs, zero_guess, together);
+  if (!s->graphs.rounds || sig != s->graphs.rounds_sig) {
+    GraphSet::drop(s->graphs.rounds);
+    if (together)
       build_rhs_graph(s, b, x, nrhs, zero_guess);
-    } else {
+    else
       build_rounds_graph(s, b, x, nrhs, zero_guess);
-    }
+    s->graphs.rounds_sig = std::move(sig);
   }
   SSAMG_CUDA(cudaGraphLaunch(s->graphs.rounds, st));
   std::vector<PcgScalars> sc((size_t)np * nrhs);
@@ -2703,7 +2757,11 @@ int run_pcg(ssamg_solver s, cudaStream_t st, ssamg_stats* stats) {
   const int np = s->nprob;
   SSAMG_CUDA(cudaMemcpyAsync(s->sc, s->sc_init, sizeof(PcgScalars) * np, cudaMemcpyDeviceToDevice, st));
   if (s->prm.use_graph) {
-    if (!s->graphs.pcg) build_pcg_graph(s);
+    if (!s->graphs.pcg || s->sig != s->graphs.pcg_sig) {
+      GraphSet::drop(s->graphs.pcg);
+      build_pcg_graph(s);
+      s->graphs.pcg_sig = s->sig;
+    }
     SSAMG_CUDA(cudaGraphLaunch(s->graphs.pcg, st));
   } else {
     long long c0 = g_ssamg_launches;
@@ -2744,6 +2802,7 @@ void run_setup(ssamg_solver s, cudaStream_t st) {
   const long long c0 = g_ssamg_launches;
   build_hierarchy(s, st);
   s->setup_launches = g_ssamg_launches - c0;
+  s->sig = graph_signature(s);
 }
 
 extern "C" int ssamg_setup(ssamg_solver s, ssamg_matrix A, void* stream) {
