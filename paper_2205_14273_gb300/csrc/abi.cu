@@ -377,7 +377,8 @@ struct ssamg_solver_s {
   std::vector<int> part_prob;  // problem of each part (empty: all 0)
   std::vector<long long> prob_cells;  // nprob + 1 first cells of each problem
   int* pb = nullptr;           // nprob + 1 level-0 block starts of each problem (device)
-  int* pbb = nullptr;          // the same in brick blocks
+  int* pbb = nullptr;          // the same in bricks of BF_64
+  int* pbf = nullptr;          // and of BF_FINAL32
   PcgCtl* ctl = nullptr;
   double* hist = nullptr;      // residual history: nprob x (max_iter + 1) squared norms
   PcgScalars* sc_init = nullptr;  // nprob starting scalars (tolerance, caps)
@@ -1027,12 +1028,40 @@ bool valid_tile(int t) {
 // Block starts of a level's launches and the first cell of every part (host
 // side of the level's device tables).
 struct LevelTables {
-  std::vector<int> blk, bblk, fblk, cs, wblk;
+  std::vector<int> blk, bblk, fblk, cs, wblk, kb[2];  // kb: BF_CYCLE32, BF_FINAL32
 };
 
 // Levels a hierarchy can have: every level halves an extent of some part, and
 // a part's extents multiply to less than 2^31.
 constexpr int kMaxLevels = 128;
+
+// Planes of a brick of the FP32 operator applies on level L (`per` resident
+// blocks an SM): a block marches its planes one after another, so a launch
+// takes as many brick times as rounds of resident blocks, and 8 planes leave
+// the last round nearly empty when the bricks are a little more than a round
+// (8 x 64^3: 1024 of 912 resident, 8 + 8 planes; with 10 planes 896 and one
+// round).  Takes the least rounds x (z + 1.5) if it saves a tenth over 8
+// planes.  Measured on 8 x 64^3 (residual 16.4 -> 11.8 us, last relaxation 27.9 ->
+// 22.5 us inside a PCG iteration; 5 uneven parts 14.5 -> 9.7 and 22.6 -> 19.5); beyond
+// four rounds the last one no longer counts.  With off-diagonals per cell the
+// kernels are bound by their seven coefficient streams, not by rounds: 8 planes
+// (2 x 96^3 refined: the solve 2.4 % slower with 10).
+int brick_planes(const Level& L, int per) {
+  auto bricks = [&](int z) {
+    long long n = 0;
+    for (const PartH& h : L.parts)
+      n += cdivll(h.n[0], SSAMG_BRICK_X) * cdivll(h.n[1], SSAMG_BRICK_Y) * cdivll(h.n[2], z);
+    return n;
+  };
+  auto cost = [&](int z) {
+    const double r = (double)bricks(z) / (SSAMG_SMS * per);
+    return (r < 4 ? std::ceil(r) : r + 0.5) * (z + 1.5);
+  };
+  int best = SSAMG_BRICK_Z;
+  for (int z = 4; z <= 16; ++z)
+    if (cost(z) < cost(best) && cost(z) < 0.9 * cost(SSAMG_BRICK_Z)) best = z;
+  return best;
+}
 
 // The host side of a level's tables: part descriptors (L.dparts), tile and
 // brick decomposition, operator-apply shape.  Copies nothing.
@@ -1124,6 +1153,21 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
     for (const DPart& dp : L.dparts)
       L.kvar = std::max(L.kvar, dp.varmask == 0 ? 0 : dp.varmask == 1u ? 1 : 2);
   }
+  // (resident blocks an SM: the launch bounds of the kernels)
+  const int per[2] = {6, 5};
+  for (int q = 0; q < 2; ++q) {
+    L.bf[q].z = L.kvar == 2 ? SSAMG_BRICK_Z : brick_planes(L, per[q]);
+    t.kb[q].assign(np + 1, 0);
+    for (int p = 0; p < np; ++p) {
+      const PartH& h = L.parts[p];
+      t.kb[q][p + 1] = t.kb[q][p] + (int)(cdivll(h.n[0], SSAMG_BRICK_X) * cdivll(h.n[1], SSAMG_BRICK_Y) *
+                                          cdivll(h.n[2], L.bf[q].z));
+    }
+    L.bf[q].n = t.kb[q][np];
+  }
+  L.bf[BF_64].z = SSAMG_BRICK_Z;
+  L.bf[BF_64].n = L.nbblk;
+  L.hfblk = t.kb[BF_FINAL32];
 }
 
 // One level's tables, copied on their own (level 0 before the coupling sums,
@@ -1140,6 +1184,8 @@ void upload_level(ssamg_solver s, Level& L, const Level* next, cudaStream_t st) 
     L.d_fblk = aalloc<int>(s->arena, np + 1);
     L.d_cellstart = aalloc<int>(s->arena, np + 1);
     L.d_wblk = aalloc<int>(s->arena, np + 1);
+    for (int q = 0; q < 2; ++q) L.bf[q].blk = aalloc<int>(s->arena, np + 1);
+    L.bf[BF_64].blk = L.d_bblk;
   }
   SSAMG_CUDA(cudaMemcpyAsync(L.d_parts, L.dparts.data(), sizeof(DPart) * np, cudaMemcpyHostToDevice, st));
   SSAMG_CUDA(cudaMemcpyAsync(L.d_blk, t.blk.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
@@ -1147,6 +1193,9 @@ void upload_level(ssamg_solver s, Level& L, const Level* next, cudaStream_t st) 
   SSAMG_CUDA(cudaMemcpyAsync(L.d_fblk, t.fblk.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
   SSAMG_CUDA(cudaMemcpyAsync(L.d_cellstart, t.cs.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
   SSAMG_CUDA(cudaMemcpyAsync(L.d_wblk, t.wblk.data(), sizeof(int) * (np + 1), cudaMemcpyHostToDevice, st));
+  for (int q = 0; q < 2; ++q)
+    SSAMG_CUDA(cudaMemcpyAsync(const_cast<int*>(L.bf[q].blk), t.kb[q].data(), sizeof(int) * (np + 1),
+                               cudaMemcpyHostToDevice, st));
 }
 
 // Every level's tables in one device block, through one pinned staging
@@ -1160,7 +1209,7 @@ void upload_levels(ssamg_solver s, cudaStream_t st) {
   for (int l = 0; l < nl; ++l) {
     level_tables(s, s->lev[l], l + 1 < nl ? &s->lev[l + 1] : nullptr, t[l]);
     const size_t np = (size_t)s->lev[l].np;
-    total += al(sizeof(DPart) * np) + 5 * al(sizeof(int) * (np + 1));
+    total += al(sizeof(DPart) * np) + 7 * al(sizeof(int) * (np + 1));
   }
   if (s->h_up_cap < total) {
     pinned_free(s->h_up);
@@ -1186,6 +1235,8 @@ void upload_levels(ssamg_solver s, cudaStream_t st) {
     L.d_fblk = (int*)put(t[l].fblk.data(), sizeof(int) * (np + 1));
     L.d_cellstart = (int*)put(t[l].cs.data(), sizeof(int) * (np + 1));
     L.d_wblk = (int*)put(t[l].wblk.data(), sizeof(int) * (np + 1));
+    for (int q = 0; q < 2; ++q) L.bf[q].blk = (int*)put(t[l].kb[q].data(), sizeof(int) * (np + 1));
+    L.bf[BF_64].blk = L.d_bblk;
   }
   SSAMG_CUDA(cudaMemcpyAsync(dev, s->h_up, o, cudaMemcpyHostToDevice, st));
 }
@@ -1934,7 +1985,7 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   s->p = (double*)padded_vector(s, sizeof(double), N, L0g, st);
   s->q = aalloc<double>(s->arena, N);
   s->zprev = aalloc<double>(s->arena, N);
-  s->partial = aalloc<double>(s->arena, 2ll * std::max(L0.nblk, L0.nbblk));
+  s->partial = aalloc<double>(s->arena, 2ll * std::max({L0.nblk, L0.nbblk, L0.bf[BF_FINAL32].n}));
   s->tres = aalloc<double>(s->arena, 2ll * s->nprob);
   s->sc = aalloc<PcgScalars>(s->arena, s->nprob);
   s->ctl = aalloc<PcgCtl>(s->arena, 1);
@@ -1955,16 +2006,21 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   }
   {
     // level-0 block and cell ranges of each problem (parts are problem-ordered)
-    std::vector<int> hpb(s->nprob + 1, L0.nblk), hpbb(s->nprob + 1, L0.nbblk);
+    std::vector<int> hpb(s->nprob + 1, L0.nblk), hpbb(s->nprob + 1, L0.nbblk),
+        hpbf(s->nprob + 1, L0.bf[BF_FINAL32].n);
     s->prob_cells.assign(s->nprob + 1, N);
     for (int p = L0.np - 1; p >= 0; --p) {
       const int k = s->part_prob.empty() ? 0 : s->part_prob[p];
       hpb[k] = L0.hblk[p];
       hpbb[k] = L0.hbblk[p];
+      hpbf[k] = L0.hfblk[p];
       s->prob_cells[k] = L0.parts[p].off;
     }
     s->pb = aalloc<int>(s->arena, s->nprob + 1);
     s->pbb = aalloc<int>(s->arena, s->nprob + 1);
+    s->pbf = aalloc<int>(s->arena, s->nprob + 1);
+    SSAMG_CUDA(cudaMemcpyAsync(s->pbf, hpbf.data(), sizeof(int) * (s->nprob + 1),
+                               cudaMemcpyHostToDevice, st));
     SSAMG_CUDA(cudaMemcpyAsync(s->pb, hpb.data(), sizeof(int) * (s->nprob + 1),
                                cudaMemcpyHostToDevice, st));
     SSAMG_CUDA(cudaMemcpyAsync(s->pbb, hpbb.data(), sizeof(int) * (s->nprob + 1),
@@ -2077,7 +2133,7 @@ int vcycle(ssamg_solver s, const double* r, double* z, cudaStream_t st, double* 
 // PCG segments.  init: r = b - A x; the first iteration is peeled so that the
 // loop body starts with the V-cycle and ends with the convergence test.
 PcgCtx pcg_ctx(ssamg_solver s) {
-  return PcgCtx{s->pb, s->pbb, s->nprob, s->sc, s->ctl, s->partial, s->hist,
+  return PcgCtx{s->pb, s->pbb, s->pbf, s->nprob, s->sc, s->ctl, s->partial, s->hist,
                 s->prm.max_iter + 1, s->any_sc ? s->any_sc : s->sc,
                 s->any_sc ? s->any_n : s->nprob};
 }
@@ -2128,6 +2184,7 @@ std::vector<char> graph_signature(ssamg_solver s) {
         L.u_val32, L.u_bits, L.u_pj, L.u_pw, L.u_pw32, L.u_rj, L.u_rw, L.u_rw32, L.uy64, L.uy32);
     put(L.nr, L.nnz, L.u_rb, L.nublk, L.tpr, L.nblk, L.nfblk, L.nbblk, L.cpt, L.bricks, L.brick_fill,
         L.kvar, L.shape, L.guard, L.x, L.b, L.r, L.t);
+    for (const BrickForm& f : L.bf) put(f.blk, f.z, f.n);
   }
   put(s->nprob, s->nL, s->chol, s->cinv, s->tail_lt, s->tail_dev, s->tail_blocks, s->tail_bar,
       s->tail_parts, s->ctail_lt);
@@ -2142,7 +2199,7 @@ std::vector<char> graph_signature(ssamg_solver s) {
     }
   }
   put(s->b, s->x, s->r, s->z, s->p, s->q, s->zprev, s->partial, s->tres, s->sc, s->sc_init, s->ctl,
-      s->hist, s->pb, s->pbb);
+      s->hist, s->pb, s->pbb, s->pbf);
   return sig;
 }
 
@@ -2370,7 +2427,7 @@ void alloc_rhs(ssamg_solver s, int R, cudaStream_t st) {
   const Level& L0 = s->lev[0];
   N.stride0 = slab(L0.N, L0.guard);  // equal to stride[0] (element counts)
   total += 7 * al(8 * N.stride0 * R);
-  N.partial_len = 2ll * std::max(L0.nblk, L0.nbblk);
+  N.partial_len = 2ll * std::max({L0.nblk, L0.nbblk, L0.bf[BF_FINAL32].n});
   total += al(8 * N.partial_len * R);
   total += al(sizeof(PcgScalars) * (size_t)s->nprob * R);
   N.hist_len = (long long)s->nprob * (s->prm.max_iter + 1);

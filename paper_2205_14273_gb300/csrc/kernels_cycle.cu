@@ -231,7 +231,8 @@ __global__ void __launch_bounds__(NT, 4) k_relax_final(LevelView<T> L, const T* 
 // ---------------------------------------------------------------------------
 // Checked 7-point operator applies over bricks (levels of shape SH_K7: entries
 // [C, -x, +x, -y, +y, -z, +z], some of them constant per part).  A block takes
-// an SSAMG_BRICK_X x _Y x _Z brick of one part and each thread marches one
+// an SSAMG_BRICK_X x _Y x z brick of one part (z planes, see brick_planes in
+// abi.cu) and each thread marches one
 // (i, j) column along z, carrying x at k-1 and k in registers: no cell
 // coordinate needs a division, and each x value comes from DRAM once (the
 // in-plane neighbours hit L1).  The operation Op supplies the per-cell inputs
@@ -241,9 +242,8 @@ __global__ void __launch_bounds__(NT, 4) k_relax_final(LevelView<T> L, const T* 
 // bitwise that of the cell-tile kernels.
 // ---------------------------------------------------------------------------
 template <class T, int KM, class Op>
-__device__ __forceinline__ void brick7(const LevelView<T>& L, const DPart& sp, const T* x,
-                                       Op& op) {
-  const int bl = (int)blockIdx.x - sp.bblk0;
+__device__ __forceinline__ void brick7(const LevelView<T>& L, const DPart& sp, int bl, int zb,
+                                       const T* x, Op& op) {
   const int bx = bl % sp.bb[0];
   const int byz = bl / sp.bb[0];
   const int by = byz % sp.bb[1];
@@ -252,8 +252,8 @@ __device__ __forceinline__ void brick7(const LevelView<T>& L, const DPart& sp, c
   const int i = bx * SSAMG_BRICK_X + (int)threadIdx.x % SSAMG_BRICK_X;
   const int j = by * SSAMG_BRICK_Y + (int)threadIdx.x / SSAMG_BRICK_X;
   if (i >= nx || j >= ny) return;
-  const int k0 = bz * SSAMG_BRICK_Z;
-  const int kend = min(k0 + SSAMG_BRICK_Z, nz);
+  const int k0 = bz * zb;
+  const int kend = min(k0 + zb, nz);
   const unsigned vm = sp.varmask;
   const T* xp0 = x + sp.off;
   const bool bw = i > 0, be = i < nx - 1, bs = j > 0, bn = j < ny - 1;
@@ -390,42 +390,42 @@ struct RelaxFinalOp {
 };
 
 template <class T, int KM>
-__global__ void __launch_bounds__(NT, brick_min_blocks<T, KM>()) k7b_residual(LevelView<T> L, const T* x, const T* b, T* r) {
+__global__ void __launch_bounds__(NT, brick_min_blocks<T, KM>()) k7b_residual(LevelView<T> L, BrickForm f, const T* x, const T* b, T* r) {
   pdl_trigger();
   __shared__ DPart sp;
-  block_part(L.bblk, L.parts, L.np, sp);
+  const int bl = (int)blockIdx.x - f.blk[block_part(f.blk, L.parts, L.np, sp)];
   __syncthreads();
   pdl_wait();
   if (L.skip && L.skip[sp.prob].done) return;  // problem already stopped
   ResidualOp<T> op{b, r};
-  brick7<T, KM>(L, sp, x, op);
+  brick7<T, KM>(L, sp, bl, f.z, x, op);
 }
 
 template <class T, int KM>
-__global__ void __launch_bounds__(NT, brick_min_blocks<T, KM>()) k7b_relax(LevelView<T> L, const T* x, const T* b, T* xo) {
+__global__ void __launch_bounds__(NT, brick_min_blocks<T, KM>()) k7b_relax(LevelView<T> L, BrickForm f, const T* x, const T* b, T* xo) {
   pdl_trigger();
   __shared__ DPart sp;
-  block_part(L.bblk, L.parts, L.np, sp);
+  const int bl = (int)blockIdx.x - f.blk[block_part(f.blk, L.parts, L.np, sp)];
   __syncthreads();
   pdl_wait();
   if (L.skip && L.skip[sp.prob].done) return;  // problem already stopped
   RelaxOp<T> op{b, L.dinv, xo};
-  brick7<T, KM>(L, sp, x, op);
+  brick7<T, KM>(L, sp, bl, f.z, x, op);
 }
 
 template <class T, int KM>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 5 : 4) k7b_relax_final(LevelView<T> L, const T* x, const T* b,
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 5 : 4) k7b_relax_final(LevelView<T> L, BrickForm f, const T* x, const T* b,
                                                       double* z, const double* rpcg,
                                                       double* zprev, int flex, double* partial) {
   pdl_trigger();
   __shared__ DPart sp;
   __shared__ double sh[NT];
-  block_part(L.bblk, L.parts, L.np, sp);
+  const int bl = (int)blockIdx.x - f.blk[block_part(f.blk, L.parts, L.np, sp)];
   __syncthreads();
   pdl_wait();
   if (L.skip && L.skip[sp.prob].done) return;  // problem already stopped
   RelaxFinalOp<T> op{b, L.dinv, z, rpcg, zprev, flex, 0.0, 0.0};
-  brick7<T, KM>(L, sp, x, op);
+  brick7<T, KM>(L, sp, bl, f.z, x, op);
   const double t0 = block_sum<NT>(op.s0, sh);
   const double t1 = block_sum<NT>(op.s1, sh);
   if (threadIdx.x == 0) {
@@ -435,16 +435,16 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 5 : 4) k7b_relax_final(Le
 }
 
 template <int KM>
-__global__ void __launch_bounds__(NT, 4) k7b_pcg_init(LevelView<double> L, const double* b,
+__global__ void __launch_bounds__(NT, 4) k7b_pcg_init(LevelView<double> L, BrickForm f, const double* b,
                                                    const double* x, double* r, double* partial) {
   pdl_trigger();
   __shared__ DPart sp;
   __shared__ double sh[NT];
-  block_part(L.bblk, L.parts, L.np, sp);
+  const int bl = (int)blockIdx.x - f.blk[block_part(f.blk, L.parts, L.np, sp)];
   __syncthreads();
   pdl_wait();
   PcgInitOp op{b, r, 0.0, 0.0};
-  brick7<double, KM>(L, sp, x, op);
+  brick7<double, KM>(L, sp, bl, f.z, x, op);
   const double s0 = block_sum<NT>(op.bb, sh);
   const double s1 = block_sum<NT>(op.rr, sh);
   if (threadIdx.x == 0) {
@@ -454,17 +454,17 @@ __global__ void __launch_bounds__(NT, 4) k7b_pcg_init(LevelView<double> L, const
 }
 
 template <int KM>
-__global__ void __launch_bounds__(NT, 4) k7b_spmv_dot(LevelView<double> L, const double* p, double* q,
+__global__ void __launch_bounds__(NT, 4) k7b_spmv_dot(LevelView<double> L, BrickForm f, const double* p, double* q,
                                                    double* partial) {
   pdl_trigger();
   __shared__ DPart sp;
   __shared__ double sh[NT];
-  block_part(L.bblk, L.parts, L.np, sp);
+  const int bl = (int)blockIdx.x - f.blk[block_part(f.blk, L.parts, L.np, sp)];
   __syncthreads();
   pdl_wait();
   if (L.skip && L.skip[sp.prob].done) return;  // problem already stopped
   SpmvDotOp op{q, 0.0};
-  brick7<double, KM>(L, sp, p, op);
+  brick7<double, KM>(L, sp, bl, f.z, p, op);
   const double t = block_sum<NT>(op.s, sh);
   if (threadIdx.x == 0) partial[blockIdx.x] = t;
 }
@@ -1235,14 +1235,14 @@ struct MatvecOp {
 
 template <int KM>
 __global__ void __launch_bounds__(NT, brick_min_blocks<double, KM>())
-    k7b_matvec(LevelView<double> L, const double* x, double* y) {
+    k7b_matvec(LevelView<double> L, BrickForm f, const double* x, double* y) {
   pdl_trigger();
   __shared__ DPart sp;
-  block_part(L.bblk, L.parts, L.np, sp);
+  const int bl = (int)blockIdx.x - f.blk[block_part(f.blk, L.parts, L.np, sp)];
   __syncthreads();
   pdl_wait();
   MatvecOp op{y};
-  brick7<double, KM>(L, sp, x, op);
+  brick7<double, KM>(L, sp, bl, f.z, x, op);
 }
 
 // ---------------------------------------------------------------------------
@@ -1822,7 +1822,8 @@ const int* partial_ranges(const Level& L, const PcgCtx& c) {
   return uses_bricks<double>(L) ? c.pbb : c.pb;
 }
 const int* final_ranges(const Level& L, const PcgCtx& c, bool fp32) {
-  return (fp32 ? uses_bricks<float>(L) : uses_bricks<double>(L)) ? c.pbb : c.pb;
+  if (fp32) return uses_bricks<float>(L) ? c.pbf : c.pb;
+  return uses_bricks<double>(L) ? c.pbb : c.pb;
 }
 
 // Blocks of a launch with nt tile blocks that come before its row jobs.  The
@@ -1878,9 +1879,10 @@ void launch_relax_final(const Level& L, const T* x, const T* b, double* z, const
   // zprev may be null (no flexible CG): pass a valid buffer and a flag
   const int flex = zprev != nullptr;
   double* zp = flex ? zprev : z;
+  constexpr int form = sizeof(T) == 4 ? BF_FINAL32 : BF_64;
   if (uses_bricks<T>(L))
     launch_k(pick_km(L.kvar, k7b_relax_final<T, 0>, k7b_relax_final<T, 1>, k7b_relax_final<T, 2>),
-             L.nbblk, NT, 0, st, L.view<T>(), x, b, z, rpcg, zp, flex, partial);
+             L.bf[form].n, NT, 0, st, L.view<T>(), L.bf[form], x, b, z, rpcg, zp, flex, partial);
   else
     SH_DISPATCH(L.shape, (launch_k(k_relax_final<T, SHV>, L.nblk, NT, 0, st, L.view<T>(), x, b, z,
                                    rpcg, zp, flex, partial)));
@@ -1906,18 +1908,20 @@ void launch_uy(const Level& L, const T* x, cudaStream_t st) {
 
 template <class T>
 void launch_residual(const Level& L, const T* x, const T* b, T* r, cudaStream_t st) {
+  constexpr int form = sizeof(T) == 4 ? BF_CYCLE32 : BF_64;
   if (uses_bricks<T>(L))
-    launch_k(pick_km(L.kvar, k7b_residual<T, 0>, k7b_residual<T, 1>, k7b_residual<T, 2>), L.nbblk, NT, 0,
-             st, L.view<T>(), x, b, r);
+    launch_k(pick_km(L.kvar, k7b_residual<T, 0>, k7b_residual<T, 1>, k7b_residual<T, 2>), L.bf[form].n, NT, 0,
+             st, L.view<T>(), L.bf[form], x, b, r);
   else
     SH_DISPATCH(L.shape, (launch_k(k_residual<T, SHV>, L.nblk, NT, 0, st, L.view<T>(), x, b, r)));
   SSAMG_LAUNCH_CHECK();
 }
 template <class T>
 void launch_relax(const Level& L, const T* x, const T* b, T* xo, cudaStream_t st) {
+  constexpr int form = sizeof(T) == 4 ? BF_CYCLE32 : BF_64;
   if (uses_bricks<T>(L))
-    launch_k(pick_km(L.kvar, k7b_relax<T, 0>, k7b_relax<T, 1>, k7b_relax<T, 2>), L.nbblk, NT, 0,
-             st, L.view<T>(), x, b, xo);
+    launch_k(pick_km(L.kvar, k7b_relax<T, 0>, k7b_relax<T, 1>, k7b_relax<T, 2>), L.bf[form].n, NT, 0,
+             st, L.view<T>(), L.bf[form], x, b, xo);
   else
     SH_DISPATCH(L.shape, (launch_k(k_relax<T, SHV>, L.nblk, NT, 0, st, L.view<T>(), x, b, xo)));
   SSAMG_LAUNCH_CHECK();
@@ -2126,8 +2130,8 @@ void launch_cast_f2d(const float* in, double* out, long long n, cudaStream_t st)
 void launch_matvec(const Level& L, const double* x, double* y, cudaStream_t st) {
   launch_uy<double>(L, x, st);
   if (uses_bricks<double>(L)) {
-    launch_k(pick_km(L.kvar, k7b_matvec<0>, k7b_matvec<1>, k7b_matvec<2>), L.nbblk, NT, 0, st,
-             L.view<double>(), x, y);
+    launch_k(pick_km(L.kvar, k7b_matvec<0>, k7b_matvec<1>, k7b_matvec<2>), L.bf[BF_64].n, NT, 0, st,
+             L.view<double>(), L.bf[BF_64], x, y);
   } else {
     int ne = L.parts[0].nent;
     for (const PartH& h : L.parts)
@@ -2147,8 +2151,8 @@ void launch_pcg_init(const Level& L, const double* b, const double* x, double* r
                      const PcgCtx& c, cudaStream_t st) {
   launch_uy<double>(L, x, st);
   if (uses_bricks<double>(L))
-    launch_k(pick_km(L.kvar, k7b_pcg_init<0>, k7b_pcg_init<1>, k7b_pcg_init<2>), L.nbblk, NT, 0,
-             st, L.view<double>(), b, x, r, c.partial);
+    launch_k(pick_km(L.kvar, k7b_pcg_init<0>, k7b_pcg_init<1>, k7b_pcg_init<2>), L.bf[BF_64].n, NT, 0,
+             st, L.view<double>(), L.bf[BF_64], b, x, r, c.partial);
   else
     SH_DISPATCH(L.shape, (launch_k(k_pcg_init<SHV>, L.nblk, NT, 0, st, L.view<double>(), b, x, r,
                                    c.partial)));
@@ -2188,8 +2192,8 @@ void launch_pcg_alpha(const Level& L, const double* p, double* q, const PcgCtx& 
                       cudaStream_t st) {
   launch_uy<double>(L, p, st);
   if (uses_bricks<double>(L))
-    launch_k(pick_km(L.kvar, k7b_spmv_dot<0>, k7b_spmv_dot<1>, k7b_spmv_dot<2>), L.nbblk, NT, 0,
-             st, L.view<double>(), p, q, c.partial);
+    launch_k(pick_km(L.kvar, k7b_spmv_dot<0>, k7b_spmv_dot<1>, k7b_spmv_dot<2>), L.bf[BF_64].n, NT, 0,
+             st, L.view<double>(), L.bf[BF_64], p, q, c.partial);
   else
     SH_DISPATCH(L.shape, (launch_k(k_pcg_spmv_dot<SHV>, L.nblk, NT, 0, st, L.view<double>(), p, q,
                                    c.partial)));
@@ -2212,8 +2216,8 @@ void launch_true_residual(const Level& L, const double* b, const double* x, doub
                           const PcgCtx& c, double* out, cudaStream_t st) {
   launch_uy<double>(L, x, st);
   if (uses_bricks<double>(L))
-    launch_k(pick_km(L.kvar, k7b_pcg_init<0>, k7b_pcg_init<1>, k7b_pcg_init<2>), L.nbblk, NT, 0,
-             st, L.view<double>(), b, x, r, c.partial);
+    launch_k(pick_km(L.kvar, k7b_pcg_init<0>, k7b_pcg_init<1>, k7b_pcg_init<2>), L.bf[BF_64].n, NT, 0,
+             st, L.view<double>(), L.bf[BF_64], b, x, r, c.partial);
   else
     SH_DISPATCH(L.shape, (launch_k(k_pcg_init<SHV>, L.nblk, NT, 0, st, L.view<double>(), b, x, r,
                                    c.partial)));

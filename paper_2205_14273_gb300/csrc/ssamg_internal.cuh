@@ -44,6 +44,7 @@
 #define SSAMG_BRICK_X 32
 #define SSAMG_BRICK_Y 8
 #define SSAMG_BRICK_Z 8
+#define SSAMG_SMS 152  // SMs of the GPU (rounds of resident blocks)
 // Fewest bricks of a level, and the least fraction of their cells inside the
 // parts, for the operator applies over bricks (see uses_bricks)
 #define SSAMG_K7_BRICKS_F32 250
@@ -152,7 +153,8 @@ struct PcgCtl {
 // brick launches) and the block partials.
 struct PcgCtx {
   const int* pb;
-  const int* pbb;  // the same in brick blocks (the level-0 brick launches' partials)
+  const int* pbb;  // the same in bricks of BF_64 and of BF_FINAL32
+  const int* pbf;
   int nprob;
   PcgScalars* sc;
   PcgCtl* ctl;
@@ -164,6 +166,15 @@ struct PcgCtx {
   const PcgScalars* any_sc;
   int any_n;
 };
+
+// Bricks of an operator apply: block starts per part (np + 1) and planes per
+// brick.  BF_CYCLE32: FP32 residual and relaxation, BF_FINAL32: the FP32 cycle's
+// last relaxation, BF_64: every FP64 apply (SSAMG_BRICK_Z planes).
+struct BrickForm {
+  const int* blk;
+  int z, n;  // planes per brick, bricks
+};
+enum { BF_CYCLE32 = 0, BF_FINAL32 = 1, BF_64 = 2, BF_FORMS = 3 };
 
 // Views passed to kernels by value.
 template <class T>
@@ -325,12 +336,14 @@ struct Level {
   int nblk = 0, nfblk = 0, nbblk = 0, nwblk = 0;
   int wcpt = 1;
   int cpt = 1;
+  BrickForm bf[BF_FORMS] = {};  // bricks of the operator applies (levels that may run over them)
   int bricks = 1; // operator applies over bricks: 0 never, 1 by the rule, 2 the table wants them
   double brick_fill = 0.0;  // cells / (bricks x brick cells): how full the level's bricks are
   int kvar = 2;   // per-cell stencil entries: 0 none, 1 only diagonals, 2 others too
   int shape = 0;  // StencilShape of the level's operator apply
   std::vector<int> hblk;  // host copy of the block starts of cell-wise launches
   std::vector<int> hbblk; // and of brick launches
+  std::vector<int> hfblk; // of BF_FINAL32
   double* coef = nullptr;
   float* coef32 = nullptr;
   long long ncoef = 0;
