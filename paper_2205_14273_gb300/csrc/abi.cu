@@ -1448,6 +1448,8 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
   }
 }
 
+bool fused_dots(ssamg_solver s);
+
 void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   ssamg_matrix A = s->A;
   const ssamg_grid g = A->g;
@@ -1984,7 +1986,7 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   s->z = aalloc<double>(s->arena, N);
   s->p = (double*)padded_vector(s, sizeof(double), N, L0g, st);
   s->q = aalloc<double>(s->arena, N);
-  s->zprev = aalloc<double>(s->arena, N);
+  s->zprev = fused_dots(s) ? nullptr : aalloc<double>(s->arena, N);
   s->partial = aalloc<double>(s->arena, 2ll * std::max({L0.nblk, L0.nbblk, L0.bf[BF_FINAL32].n}));
   s->tres = aalloc<double>(s->arena, 2ll * s->nprob);
   s->sc = aalloc<PcgScalars>(s->arena, s->nprob);
@@ -2030,13 +2032,21 @@ void build_hierarchy(ssamg_solver s, cudaStream_t st) {
   s->ready = true;
 }
 
-// One V(1,1) cycle z = M r (r, z: FP64 level-0 vectors).
-// One V(1,1) cycle z = M r.  With `dots` set, the last post-relaxation also
-// produces the PCG's r.z (and r.zprev) block partials in `dots` and the
-// function returns their block count (0: not fused, compute them apart).
+// Whether the cycle's last relaxation runs as a kernel of its own (not inside a
+// tail), and can form the PCG's dot partials; z then keeps the previous z for
+// flexible CG, else zprev does.
+bool fused_dots(ssamg_solver s) {
+  const int Lc = (int)s->lev.size() - 1;
+  return Lc > 0 && (s->ctail_lt >= 1 || s->tail_lt != 0);
+}
+
+// One V(1,1) cycle z = M r (r, z: FP64 level-0 vectors).  With `dots` set, the
+// last post-relaxation also produces the PCG's r.z and (flexible CG) r.zprev
+// block partials in `dots` and the function returns their block count (0: not
+// fused, compute them apart).
 template <class T>
 int enqueue_vcycle(ssamg_solver s, const double* r_in, double* z_out, cudaStream_t st,
-                   double* dots = nullptr, double* zprev = nullptr) {
+                   double* dots = nullptr) {
   auto& Ls = s->lev;
   const int Lc = (int)Ls.size() - 1;
   const bool is_f = sizeof(T) == sizeof(float);
@@ -2114,7 +2124,7 @@ int enqueue_vcycle(ssamg_solver s, const double* r_in, double* z_out, cudaStream
     if (l == 0 && (dots || is_f)) {
       // straight into the FP64 z (and the PCG dot partials when asked)
       double* part = dots ? dots : s->partial;
-      launch_relax_final<T>(Ls[0], xc, bl, z_out, r_in, dots ? zprev : nullptr, part, st);
+      launch_relax_final<T>(Ls[0], xc, bl, z_out, r_in, dots && s->prm.flexible, part, st);
       return dots ? Ls[0].nblk : 0;
     }
     T* out = (l == 0) ? (T*)z_out : (T*)Ls[l].t;
@@ -2124,10 +2134,9 @@ int enqueue_vcycle(ssamg_solver s, const double* r_in, double* z_out, cudaStream
   return 0;
 }
 
-int vcycle(ssamg_solver s, const double* r, double* z, cudaStream_t st, double* dots = nullptr,
-           double* zprev = nullptr) {
-  if (s->prm.precision == 1) return enqueue_vcycle<float>(s, r, z, st, dots, zprev);
-  return enqueue_vcycle<double>(s, r, z, st, dots, zprev);
+int vcycle(ssamg_solver s, const double* r, double* z, cudaStream_t st, double* dots = nullptr) {
+  if (s->prm.precision == 1) return enqueue_vcycle<float>(s, r, z, st, dots);
+  return enqueue_vcycle<double>(s, r, z, st, dots);
 }
 
 // PCG segments.  init: r = b - A x; the first iteration is peeled so that the
@@ -2140,7 +2149,7 @@ PcgCtx pcg_ctx(ssamg_solver s) {
 
 void enqueue_pcg_head(ssamg_solver s, cudaGraphConditionalHandle h, int use_h, cudaStream_t st) {
   Level& L0 = s->lev[0];
-  double* zp = s->prm.flexible ? s->zprev : nullptr;
+  double* zp = s->prm.flexible && !fused_dots(s) ? s->zprev : nullptr;
   const PcgCtx c = pcg_ctx(s);
   SkipScope skip(s->sc);
   launch_pcg_init(L0, s->b, s->x, s->r, c, st);
@@ -2156,7 +2165,7 @@ void enqueue_pcg_body(ssamg_solver s, cudaGraphConditionalHandle h, int use_h, c
   // the cycle's last kernel also forms r.z (and r.zprev) for beta
   const PcgCtx c = pcg_ctx(s);
   SkipScope skip(s->sc);
-  const int npart = vcycle(s, s->r, s->z, st, s->partial, zp);
+  const int npart = vcycle(s, s->r, s->z, st, s->partial);
   if (npart > 0)  // the last relaxation writes partials per block of its tiles
     launch_pcg_beta_from_partials(L0, s->z, s->p, c, final_ranges(L0, c, s->prm.precision == 1), st);
   else
@@ -2426,7 +2435,8 @@ void alloc_rhs(ssamg_solver s, int R, cudaStream_t st) {
   }
   const Level& L0 = s->lev[0];
   N.stride0 = slab(L0.N, L0.guard);  // equal to stride[0] (element counts)
-  total += 7 * al(8 * N.stride0 * R);
+  const int nv = fused_dots(s) ? 6 : 7;  // zprev only where the cycle does not form the dots
+  total += nv * al(8 * N.stride0 * R);
   N.partial_len = 2ll * std::max({L0.nblk, L0.nbblk, L0.bf[BF_FINAL32].n});
   total += al(8 * N.partial_len * R);
   total += al(sizeof(PcgScalars) * (size_t)s->nprob * R);
@@ -2458,7 +2468,7 @@ void alloc_rhs(ssamg_solver s, int R, cudaStream_t st) {
     }
   }
   double** pv[7] = {&N.pb, &N.px, &N.pr, &N.pz, &N.pp, &N.pq, &N.pzprev};
-  for (double** q : pv) *q = (double*)take(8 * N.stride0 * R) + L0.guard;
+  for (int v = 0; v < nv; ++v) *pv[v] = (double*)take(8 * N.stride0 * R) + L0.guard;
   N.partial = (double*)take(8 * N.partial_len * R);
   N.sc = (PcgScalars*)take(sizeof(PcgScalars) * (size_t)s->nprob * R);
   N.hist = (double*)take(8 * N.hist_len * R);
@@ -2515,7 +2525,7 @@ void use_rhs(ssamg_solver s, int j) {
   s->z = M.pz + o0;
   s->p = M.pp + o0;
   s->q = M.pq + o0;
-  s->zprev = M.pzprev + o0;
+  s->zprev = M.pzprev ? M.pzprev + o0 : nullptr;
   s->partial = M.partial + j * M.partial_len;
   s->hist = M.hist + j * M.hist_len;
   s->sc = M.sc + (long long)j * s->nprob;
@@ -2603,8 +2613,8 @@ int enqueue_vcycle_rhs(ssamg_solver s, bool dots, cudaStream_t st) {
     each([&] { launch_prolong_u<T>(Ls[l], e_of(l), (const T*)Ls[l].x, (T*)Ls[l].r, st); });
     if (l == 0 && (dots || is_f)) {
       each([&] {
-        launch_relax_final<T>(Ls[0], (const T*)Ls[0].r, b0(), s->z, s->r,
-                              dots ? s->zprev : nullptr, s->partial, st);
+        launch_relax_final<T>(Ls[0], (const T*)Ls[0].r, b0(), s->z, s->r, dots && s->prm.flexible,
+                              s->partial, st);
       });
       return dots ? Ls[0].nblk : 0;
     }
@@ -2641,7 +2651,8 @@ void enqueue_pcg_head_rhs(ssamg_solver s, cudaGraphConditionalHandle h, cudaStre
   for (int j = 0; j < R; ++j) {
     use_rhs(s, j);
     const PcgCtx c = pcg_ctx(s);
-    launch_pcg_start(L0, s->r, s->z, s->p, s->prm.flexible ? s->zprev : nullptr, c, st);
+    launch_pcg_start(L0, s->r, s->z, s->p,
+                     s->prm.flexible && !fused_dots(s) ? s->zprev : nullptr, c, st);
     launch_pcg_alpha(L0, s->p, s->q, c, st);
     launch_pcg_update(L0, s->p, s->q, s->x, s->r, c, h, 1, st);
   }
@@ -3319,12 +3330,12 @@ double time_kernel_us(ssamg_solver s, int kernel, int level, int reps, cudaStrea
       case 9:  // the cycle's last post-relaxation as the PCG runs it (FP64 z, dot partials)
         if (f)
           launch_relax_final<float>(s->lev[0], (const float*)s->lev[0].r,
-                                    (const float*)s->lev[0].b, s->z, s->r, s->prm.flexible ? s->zprev : nullptr,
+                                    (const float*)s->lev[0].b, s->z, s->r, s->prm.flexible,
                                     s->partial, cs);
         else
           launch_relax_final<double>(s->lev[0], (const double*)s->lev[0].r,
                                      (const double*)s->lev[0].b, s->z, s->r,
-                                     s->prm.flexible ? s->zprev : nullptr, s->partial, cs);
+                                     s->prm.flexible, s->partial, cs);
         break;
       case 8:  // the PCG's vector steps: beta, p = z + beta p, alpha, x and r updates
         launch_pcg_beta_from_partials(s->lev[0], s->z, s->p, pcg_ctx(s),

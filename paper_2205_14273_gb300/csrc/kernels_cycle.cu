@@ -189,13 +189,14 @@ __global__ void __launch_bounds__(NT, rhs_min_blocks<T, SH>()) k_cycle_r(LevelVi
 
 // Last post-relaxation of the cycle: t = x + omega M^-1 (b - A x) written as
 // the FP64 preconditioned residual z, with the block partials of r.z and
-// r.zprev (flexible CG; zprev then takes z) for the PCG's beta.
+// (flexible CG) r.zprev for the PCG's beta.  zprev, the last cycle's z, is what
+// z still holds: read before its store, so it needs no copy of its own (16.8
+// MB less written and held a cycle at 2.1M cells).
 template <class T, int SH>
 __global__ void __launch_bounds__(NT, 4) k_relax_final(LevelView<T> L, const T* x,
                                                        const T* b,
                                                        double* z,
-                                                       const double* rpcg,
-                                                       double* zprev, int flex,
+                                                       const double* rpcg, int flex,
                                                        double* partial) {
   pdl_trigger();
   __shared__ DPart sp;
@@ -207,18 +208,13 @@ __global__ void __launch_bounds__(NT, 4) k_relax_final(LevelView<T> L, const T* 
   double s0 = 0.0, s1 = 0.0;
   TILE_LOOP(c, sp) {
     const int g = sp.off + c;
-    // the FP64 operands are fetched with the stencil's, not after it (zprev
-    // is a valid buffer even without flexible CG: z itself, read before its
-    // store and then unused)
+    // the FP64 operands are fetched with the stencil's, not after it
     const double rv = rpcg[g];
-    const double zo = zprev[g];
+    const double zo = z[g];
     const double zv = (double)fma(L.dinv[g], b[g] - apply_A_sh<SH>(L, sp, x, c), x[g]);
     z[g] = zv;
     s0 = fma(rv, zv, s0);
-    if (flex) {
-      s1 = fma(rv, zo, s1);
-      zprev[g] = zv;
-    }
+    if (flex) s1 = fma(rv, zo, s1);
   }
   const double t0 = block_sum<NT>(s0, sh);
   const double t1 = block_sum<NT>(s1, sh);
@@ -370,22 +366,18 @@ struct RelaxFinalOp {
   const T* dinv;
   double* z;
   const double* rpcg;
-  double* zprev;
   int flex;
   double s0, s1;
   struct In {
     T b, d;
     double r, zo;
   };
-  __device__ In load(int g) const { return In{b[g], dinv[g], rpcg[g], zprev[g]}; }
+  __device__ In load(int g) const { return In{b[g], dinv[g], rpcg[g], z[g]}; }
   __device__ void apply(int g, T ax, T xg, In in) {
     const double zv = (double)fma(in.d, in.b - ax, xg);
     z[g] = zv;
     s0 = fma(in.r, zv, s0);
-    if (flex) {
-      s1 = fma(in.r, in.zo, s1);
-      zprev[g] = zv;
-    }
+    if (flex) s1 = fma(in.r, in.zo, s1);
   }
 };
 
@@ -415,8 +407,8 @@ __global__ void __launch_bounds__(NT, brick_min_blocks<T, KM>()) k7b_relax(Level
 
 template <class T, int KM>
 __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 5 : 4) k7b_relax_final(LevelView<T> L, BrickForm f, const T* x, const T* b,
-                                                      double* z, const double* rpcg,
-                                                      double* zprev, int flex, double* partial) {
+                                                      double* z, const double* rpcg, int flex,
+                                                      double* partial) {
   pdl_trigger();
   __shared__ DPart sp;
   __shared__ double sh[NT];
@@ -424,7 +416,7 @@ __global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 5 : 4) k7b_relax_final(Le
   __syncthreads();
   pdl_wait();
   if (L.skip && L.skip[sp.prob].done) return;  // problem already stopped
-  RelaxFinalOp<T> op{b, L.dinv, z, rpcg, zprev, flex, 0.0, 0.0};
+  RelaxFinalOp<T> op{b, L.dinv, z, rpcg, flex, 0.0, 0.0};
   brick7<T, KM>(L, sp, bl, f.z, x, op);
   const double t0 = block_sum<NT>(op.s0, sh);
   const double t1 = block_sum<NT>(op.s1, sh);
@@ -1875,17 +1867,14 @@ void launch_relax0_u_first(const Level& L, const double* r64, T* b0, T* x, cudaS
 }
 template <class T>
 void launch_relax_final(const Level& L, const T* x, const T* b, double* z, const double* rpcg,
-                        double* zprev, double* partial, cudaStream_t st) {
-  // zprev may be null (no flexible CG): pass a valid buffer and a flag
-  const int flex = zprev != nullptr;
-  double* zp = flex ? zprev : z;
+                        int flex, double* partial, cudaStream_t st) {
   constexpr int form = sizeof(T) == 4 ? BF_FINAL32 : BF_64;
   if (uses_bricks<T>(L))
     launch_k(pick_km(L.kvar, k7b_relax_final<T, 0>, k7b_relax_final<T, 1>, k7b_relax_final<T, 2>),
-             L.bf[form].n, NT, 0, st, L.view<T>(), L.bf[form], x, b, z, rpcg, zp, flex, partial);
+             L.bf[form].n, NT, 0, st, L.view<T>(), L.bf[form], x, b, z, rpcg, flex, partial);
   else
     SH_DISPATCH(L.shape, (launch_k(k_relax_final<T, SHV>, L.nblk, NT, 0, st, L.view<T>(), x, b, z,
-                                   rpcg, zp, flex, partial)));
+                                   rpcg, flex, partial)));
   SSAMG_LAUNCH_CHECK();
 }
 template <class T>
@@ -2096,7 +2085,7 @@ void launch_coarse_inverse(int n, const double* Lfac, double* inv, cudaStream_t 
   template void launch_prolong_u<T>(const Level&, const T*, const T*, T*, cudaStream_t);   \
   template void launch_relax0_u_first<T>(const Level&, const double*, T*, T*, cudaStream_t); \
   template void launch_relax_final<T>(const Level&, const T*, const T*, double*, const double*, \
-                                      double*, double*, cudaStream_t);                     \
+                                      int, double*, cudaStream_t);                         \
   template void launch_uy<T>(const Level&, const T*, cudaStream_t);                        \
   template void launch_vtail<T>(const TailLevel<T>*, int, const double*, int, int, int,      \
                                 TailBarrier*, cudaStream_t, int);                          \

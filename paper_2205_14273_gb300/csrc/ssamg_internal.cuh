@@ -522,7 +522,7 @@ template <class T>
 void launch_relax0_u_first(const Level& L, const double* r64, T* b0, T* x, cudaStream_t st);
 template <class T>
 void launch_relax_final(const Level& L, const T* x, const T* b, double* z, const double* rpcg,
-                        double* zprev, double* partial, cudaStream_t st);
+                        int flex, double* partial, cudaStream_t st);
 // row-job setup data of L's couplings: P rows (L.u_pj set) and restriction
 // rows from the level above Fp (L.u_rj set)
 // longest U row of every level (maxrow[l], zeroed by the caller), and u_rb of
