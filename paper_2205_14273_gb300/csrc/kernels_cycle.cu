@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(NT, brick_min_blocks<T, KM>()) k7b_relax(Level
 }
 
 template <class T, int KM>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 5 : 4) k7b_relax_final(LevelView<T> L, BrickForm f, const T* x, const T* b,
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 && KM < 2 ? 5 : 4) k7b_relax_final(LevelView<T> L, BrickForm f, const T* x, const T* b,
                                                       double* z, const double* rpcg, int flex,
                                                       double* partial) {
   pdl_trigger();
