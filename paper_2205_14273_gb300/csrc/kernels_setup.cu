@@ -1237,12 +1237,63 @@ __global__ void __launch_bounds__(1024) k_scan_sums(int* __restrict__ sums, int 
   if (threadIdx.x == 0) sums[nb] = carry;
 }
 
+// Up to SCAN_ONE_ITEMS items by one block of 1024 threads, 4096 at a time with a
+// running carry: one launch of 3-4 us where the two-launch form takes 9 (the
+// coupling chain of a set-up holds two scans per level).
+constexpr int SCAN_ONE_ITEMS = 16384;
+__global__ void __launch_bounds__(1024) k_scan_one(int* __restrict__ data, int n) {
+  __shared__ int wsum[32];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int carry = 0;
+  for (int base = 0; base < n; base += 4096) {
+    int v[4], own = 0;
+    const int t0 = base + 4 * (int)threadIdx.x;
+    if (t0 + 4 <= n) {
+      const int4 q = *reinterpret_cast<const int4*>(data + t0);  // (data: 256-byte aligned)
+      v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) v[u] = t0 + u < n ? data[t0 + u] : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) own += v[u];
+    int x = own;
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    if (lane == 31) wsum[w] = x;
+    __syncthreads();
+    if (w == 0) {
+      int s = wsum[lane];
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, s, o);
+        if (lane >= o) s += y;
+      }
+      wsum[lane] = s;
+    }
+    __syncthreads();
+    int e = carry + x - own + (w > 0 ? wsum[w - 1] : 0);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (t0 + u < n) data[t0 + u] = e;
+      e += v[u];
+    }
+    carry += wsum[31];
+    __syncthreads();
+  }
+  if (threadIdx.x == 0) data[n] = carry;
+}
+
 // Block b scans items [b SCAN_ITEMS, (b+1) SCAN_ITEMS) in parallel (four
 // consecutive items per thread, shuffle scan of the thread sums, then the
-// warp sums) and adds the block's offset sums[b] (0 without sums: the
-// single-block case).  The last block writes the total to data[n].
+// warp sums) and adds the sum of the blocks before it: sums[b] when the sums
+// are scanned, else it adds them itself (at most SCAN_OWN_BLOCKS blocks; a
+// launch less).  The last block writes the total to data[n].
+constexpr int SCAN_OWN_BLOCKS = 1024;
 __global__ void __launch_bounds__(NT) k_scan_apply(int* __restrict__ data, long long n,
-                                                   const int* __restrict__ sums, int nb) {
+                                                   const int* __restrict__ sums, int scanned,
+                                                   int nb) {
   static_assert(SCAN_ITEMS == 4 * NT, "four items per thread");
   __shared__ int sh[SCAN_ITEMS];
   __shared__ int wsum[NT / 32];
@@ -1269,7 +1320,18 @@ __global__ void __launch_bounds__(NT) k_scan_apply(int* __restrict__ data, long 
     if (lane < NT / 32) wsum[lane] = v;  // inclusive warp totals
   }
   __syncthreads();
-  const int off0 = sums ? sums[blockIdx.x] : 0;
+  __shared__ int before;
+  if (threadIdx.x == 0) before = 0;
+  __syncthreads();
+  int part = 0;
+  if (scanned)
+    part = threadIdx.x == 0 ? sums[blockIdx.x] : 0;
+  else
+    for (int t = threadIdx.x; t < (int)blockIdx.x; t += NT) part += sums[t];
+  part = __reduce_add_sync(0xffffffffu, part);
+  if (lane == 0 && part) atomicAdd(&before, part);
+  __syncthreads();
+  const int off0 = before;
   const int e = off0 + x - own + (w > 0 ? wsum[w - 1] : 0);
   sh[t4] = e;
   sh[t4 + 1] = e + a0;
@@ -1278,8 +1340,7 @@ __global__ void __launch_bounds__(NT) k_scan_apply(int* __restrict__ data, long 
   __syncthreads();
   for (int t = threadIdx.x; t < SCAN_ITEMS; t += NT)
     if (base + t < n) data[base + t] = sh[t];
-  if (blockIdx.x == nb - 1 && threadIdx.x == 0)
-    data[n] = sums ? sums[nb] : wsum[NT / 32 - 1];
+  if (blockIdx.x == nb - 1 && threadIdx.x == 0) data[n] = off0 + wsum[NT / 32 - 1];
 }
 
 inline int cdiv(long long a, long long b) { return (int)((a + b - 1) / b); }
@@ -1624,17 +1685,20 @@ void launch_scan(int* data, long long n, int* tmp, cudaStream_t st) {
     SSAMG_CUDA(cudaMemsetAsync(data, 0, sizeof(int), st));
     return;
   }
-  int nb = cdiv(n, SCAN_ITEMS);
-  if (nb == 1) {  // one block scans it all
-    k_scan_apply<<<1, NT, 0, st>>>(data, n, nullptr, 1);
+  if (n <= SCAN_ONE_ITEMS) {
+    k_scan_one<<<1, 1024, 0, st>>>(data, (int)n);
     SSAMG_LAUNCH_CHECK();
     return;
   }
+  const int nb = cdiv(n, SCAN_ITEMS);
   k_scan_reduce<<<nb, NT, 0, st>>>(data, n, tmp);
   SSAMG_LAUNCH_CHECK();
-  k_scan_sums<<<1, 1024, 0, st>>>(tmp, nb);
-  SSAMG_LAUNCH_CHECK();
-  k_scan_apply<<<nb, NT, 0, st>>>(data, n, tmp, nb);
+  const int scanned = nb > SCAN_OWN_BLOCKS;
+  if (scanned) {
+    k_scan_sums<<<1, 1024, 0, st>>>(tmp, nb);
+    SSAMG_LAUNCH_CHECK();
+  }
+  k_scan_apply<<<nb, NT, 0, st>>>(data, n, tmp, scanned, nb);
   SSAMG_LAUNCH_CHECK();
 }
 
