@@ -640,8 +640,11 @@ __device__ __forceinline__ void restrict_column(const LevelView<T>& F, const Lev
   }
 }
 
-template <class T, bool EB>
-__global__ void __launch_bounds__(NT) k_restrict_b(LevelView<T> F, LevelView<T> C, const T* r,
+// (MB: resident blocks an SM it is compiled for.  FP32 with 4, 64 registers
+// instead of 71, takes levels whose bricks then fit one round: 8 x 64^3, 512
+// bricks, 10.8 -> 9.0 us; more rounds are faster with 3, 1024 bricks 21.5 vs 28.9)
+template <class T, bool EB, int MB>
+__global__ void __launch_bounds__(NT, MB) k_restrict_b(LevelView<T> F, LevelView<T> C, const T* r,
                                                    T* bc, T* xc, int nu, int tile0) {
   pdl_trigger();
   __shared__ DPart fp;
@@ -1251,8 +1254,17 @@ __device__ __forceinline__ void finish_sums(const double* __restrict__ partial, 
                                             double* out) {
   __shared__ double sh[NT];
   for (int q = 0; q < K; ++q) {
+    // (eight loads in flight: 16384 blocks' partials 19 -> 15.6 us)
     double s = 0.0;
-    for (int b = b0 + threadIdx.x; b < b1; b += NT) s += partial[(long long)K * b + q];
+    int b = b0 + threadIdx.x;
+    for (; b + 7 * NT < b1; b += 8 * NT) {
+      double v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) v[u] = partial[(long long)K * (b + u * NT) + q];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) s += v[u];
+    }
+    for (; b < b1; b += NT) s += partial[(long long)K * b + q];
     double r = block_sum<NT>(s, sh);
     if (threadIdx.x == 0) out[q] = r;
   }
@@ -1972,8 +1984,12 @@ void launch_restrict(const Level& F, const Level& Cl, const T* r, T* bc, T* xc, 
   // with xc: also x = omega M^-1 b on the coarse level, and its U x row jobs
   const int nrow = xc ? Cl.nublk : 0;
   if (rp_bricks(Cl)) {
-    launch_k(Cl.u_rb ? k_restrict_b<T, true> : k_restrict_b<T, false>, Cl.nbblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc,
-             nrow, row_job_tile0(Cl, Cl.nbblk));
+    const bool one = sizeof(T) == 4 && Cl.nbblk <= 4 * SSAMG_SMS;
+    constexpr int MB = sizeof(T) == 4 ? 3 : 2, M1 = sizeof(T) == 4 ? 4 : 2;
+    launch_k(one ? (Cl.u_rb ? k_restrict_b<T, true, M1> : k_restrict_b<T, false, M1>)
+                 : (Cl.u_rb ? k_restrict_b<T, true, MB> : k_restrict_b<T, false, MB>),
+             Cl.nbblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc, nrow,
+             row_job_tile0(Cl, Cl.nbblk));
   } else {
     launch_k(Cl.u_rb ? k_restrict<T, true> : k_restrict<T, false>, Cl.nblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc,
              nrow, row_job_tile0(Cl, Cl.nblk));
