@@ -766,7 +766,7 @@ __device__ __forceinline__ void prolong_column(const LevelView<T>& F, const DPar
 }
 
 template <class T, bool EB>
-__global__ void __launch_bounds__(NT) k_prolong_ub(LevelView<T> F, const T* ec, const T* xin,
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 ? 8 : 6) k_prolong_ub(LevelView<T> F, const T* ec, const T* xin,
                                                    T* xout, int nu, int tile0) {
   pdl_trigger();
   __shared__ DPart fp;
