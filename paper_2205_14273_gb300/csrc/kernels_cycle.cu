@@ -640,9 +640,10 @@ __device__ __forceinline__ void restrict_column(const LevelView<T>& F, const Lev
   }
 }
 
-// (MB: resident blocks an SM it is compiled for.  FP32 with 4, 64 registers
-// instead of 71, takes levels whose bricks then fit one round: 8 x 64^3, 512
-// bricks, 10.8 -> 9.0 us; more rounds are faster with 3, 1024 bricks 21.5 vs 28.9)
+// (MB: resident blocks an SM it is compiled for.  With 4 (64 registers instead of
+// 71, FP64 108 and some spilled) it takes levels whose bricks then fit one round:
+// 8 x 64^3, 512 bricks, FP32 10.8 -> 9.0 us, FP64 20.2 -> 15.1; more rounds are faster
+// with 3, FP32 1024 bricks 21.5 vs 28.9)
 template <class T, bool EB, int MB>
 __global__ void __launch_bounds__(NT, MB) k_restrict_b(LevelView<T> F, LevelView<T> C, const T* r,
                                                    T* bc, T* xc, int nu, int tile0) {
@@ -1984,9 +1985,9 @@ void launch_restrict(const Level& F, const Level& Cl, const T* r, T* bc, T* xc, 
   // with xc: also x = omega M^-1 b on the coarse level, and its U x row jobs
   const int nrow = xc ? Cl.nublk : 0;
   if (rp_bricks(Cl)) {
-    const bool one = sizeof(T) == 4 && Cl.nbblk <= 4 * SSAMG_SMS;
-    constexpr int MB = sizeof(T) == 4 ? 3 : 2, M1 = sizeof(T) == 4 ? 4 : 2;
-    launch_k(one ? (Cl.u_rb ? k_restrict_b<T, true, M1> : k_restrict_b<T, false, M1>)
+    const bool one = Cl.nbblk <= 4 * SSAMG_SMS;
+    constexpr int MB = sizeof(T) == 4 ? 3 : 2;
+    launch_k(one ? (Cl.u_rb ? k_restrict_b<T, true, 4> : k_restrict_b<T, false, 4>)
                  : (Cl.u_rb ? k_restrict_b<T, true, MB> : k_restrict_b<T, false, MB>),
              Cl.nbblk + nrow, NT, 0, st, F.view<T>(), Cl.view<T>(), r, bc, xc, nrow,
              row_job_tile0(Cl, Cl.nbblk));
