@@ -760,6 +760,21 @@ void launch_ctail_columns(const CTailArgs& a, double* dense, cudaStream_t st) {
   SSAMG_LAUNCH_CHECK();
 }
 
+// Dynamic shared memory k_ctail<T> is allowed on device dev: at least smem.  The
+// attribute belongs to the function, not to a launch, so it is never lowered: a
+// solver set up later with a smaller tail must not cut off the launches of one
+// set up before.  (Called with ctail_prepare's lock.)
+template <class T>
+cudaError_t ctail_allow(int dev, long long smem) {
+  static std::map<int, long long> allowed;
+  long long& a = allowed[dev];
+  if (smem <= a) return cudaSuccess;
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (e == cudaSuccess) a = smem;
+  return e;
+}
+
 template <class T>
 bool ctail_prepare(int nc, long long smem) {
   // the answer per device and (nc, smem) is kept: the occupancy query costs
@@ -772,26 +787,19 @@ bool ctail_prepare(int nc, long long smem) {
     return false;
   }
   const auto key = std::make_tuple(dev, nc, smem);
-  {
-    std::lock_guard<std::mutex> lock(mu);
-    auto it = known.find(key);
-    if (it != known.end()) {
-      if (it->second)
-        SSAMG_CUDA(cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-      return it->second;
-    }
-  }
-  const bool ok = ctail_query<T>(nc, smem);
   std::lock_guard<std::mutex> lock(mu);
-  known[key] = ok;
-  return ok;
+  auto it = known.find(key);
+  if (it != known.end()) return it->second;
+  if (ctail_allow<T>(dev, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return known[key] = false;
+  }
+  return known[key] = ctail_query<T>(nc, smem);
 }
 
 template <class T>
 bool ctail_query(int nc, long long smem) {
   if (cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
           cudaSuccess) {
     cudaGetLastError();
     return false;
