@@ -1200,7 +1200,7 @@ __global__ void k_cast_f2d(const float* in, double* out, int n) {
 // 52.9 -> 39.1 us with the U x launch before it, of 25 us for the FP64 pipe (7
 // multiply-adds a cell).
 template <int K>
-__global__ void __launch_bounds__(NT, K == 15 ? 2 : K == 27 ? 3 : 4)
+__global__ void __launch_bounds__(NT, K == 15 ? 2 : 4)
     k_matvec(LevelView<double> L, const double* x, double* y) {
   pdl_trigger();
   __shared__ DPart sp;
@@ -1594,8 +1594,8 @@ __global__ void __launch_bounds__(NT) k_exp(int n, const double* gg, double* kap
   if (c < n) kap[c] = exp(gg[c]);
 }
 
-// dL/dg at cell c = (i, j, k) from its six faces, a division each: the form
-// for coefficients beyond the shared-face kernel's range.
+// dL/dg at cell c = (i, j, k) from its six faces, a division each: the form of
+// small boxes and for coefficients beyond the shared-face kernel's range.
 __device__ __forceinline__ double dg_cell(const DPart& sp, const double* kap, const double* lam,
                                           const double* x, int c, int i, int j, int k) {
   const double kc = kap[c];
@@ -1620,6 +1620,25 @@ __device__ __forceinline__ double dg_cell(const DPart& sp, const double* kap, co
   face(k > 0, -sz);
   face(k < sp.n[2] - 1, sz);
   return kc * acc;
+}
+
+// A thread per cell: boxes below SSAMG_DG_CELLS cells, whose few blocks leave the
+// FP64 pipe idle, so that the shared-face form's barriers cost more than its
+// instructions save (passes one after another: 32^3 12.8 us, host-bound, vs 23.6;
+// 40^3 43 vs 27 us).
+__global__ void __launch_bounds__(NT) k_diffusion_exp_cells(LevelView<double> L, const double* kap,
+                                                            const double* lam, const double* x,
+                                                            double* dg) {
+  pdl_trigger();
+  __shared__ DPart sp;
+  stage_part(sp, L.parts);
+  __syncthreads();
+  pdl_wait();
+  const int c = blockIdx.x * NT + threadIdx.x;
+  if (c >= sp.ncell) return;
+  int i, j, k;
+  cell_coords(sp, c, i, j, k);
+  dg[c] = dg_cell(sp, kap, lam, x, c, i, j, k);
 }
 
 // 1 / s for s in [2^-200, 2^200] (else `bad` is set and the value is not
@@ -1650,7 +1669,8 @@ __device__ __forceinline__ double rcp_fp64(double s, bool& bad) {
 // took 102 FP64 instructions a cell, here ~40 (9 per face and its reciprocal
 // without conversions; the exponential before it another 15).  128^3: 455 ->
 // 235 us with the exponential.
-// A block takes a GX x GY column of cells, GZ planes of it: the plane's kappa,
+// A block takes a GX x GY column of cells, `planes` of it (up to GZ, fewer where
+// the box then has less than four blocks an SM): the plane's kappa,
 // kappa^2, lambda and x with a halo in shared memory (double-buffered along
 // z), t of the faces towards +x and +y through shared memory, that towards
 // +z kept in a register for the next plane.  The faces between two blocks are
@@ -1662,7 +1682,7 @@ __global__ void __launch_bounds__(NT) k_diffusion_exp_gradient(LevelView<double>
                                                                const double* kap,
                                                                const double* lam,
                                                                const double* x,
-                                                               double* dg, int nbx, int nby) {
+                                                               double* dg, int nbx, int nby, int planes) {
   static_assert(GX * GY == NT && GX == 32, "a warp per row");
   pdl_trigger();
   __shared__ DPart sp;
@@ -1674,8 +1694,8 @@ __global__ void __launch_bounds__(NT) k_diffusion_exp_gradient(LevelView<double>
   pdl_wait();
   const int nx = sp.n[0], ny = sp.n[1], nz = sp.n[2], nxy = nx * ny;
   const int bx = blockIdx.x % nbx, byz = blockIdx.x / nbx;
-  const int i0 = bx * GX, j0 = (byz % nby) * GY, k0 = (byz / nby) * GZ;
-  const int kend = min(k0 + GZ, nz);
+  const int i0 = bx * GX, j0 = (byz % nby) * GY, k0 = (byz / nby) * planes;
+  const int kend = min(k0 + planes, nz);
   const int t = threadIdx.x, ti = t % GX, tj = t / GX;
   const int i = i0 + ti, j = j0 + tj;
   const bool in = i < nx && j < ny;
@@ -2243,9 +2263,18 @@ void launch_diffusion_exp_gradient(const Level& L, const double* g, const double
   const int n = (int)L.parts[0].ncell;
   launch_k(k_exp, cdiv(n, NT), NT, 0, st, n, g, kap);
   SSAMG_LAUNCH_CHECK();
+  if (n < SSAMG_DG_CELLS) {
+    launch_k(k_diffusion_exp_cells, cdiv(n, NT), NT, 0, st, L.view<double>(), (const double*)kap, lam,
+             x, dg);
+    SSAMG_LAUNCH_CHECK();
+    return;
+  }
   const int* e = L.parts[0].n;
   const int nbx = cdiv(e[0], GX), nby = cdiv(e[1], GY);
-  launch_k(k_diffusion_exp_gradient, nbx * nby * cdiv(e[2], GZ), NT, 0, st, L.view<double>(),
-           (const double*)kap, lam, x, dg, nbx, nby);
+  // as many planes as leave four blocks an SM
+  const long long cols = (long long)nbx * nby;
+  const int planes = (int)std::max(1ll, std::min((long long)GZ, cols * e[2] / (4 * SSAMG_SMS)));
+  launch_k(k_diffusion_exp_gradient, (int)(cols * cdiv(e[2], planes)), NT, 0, st, L.view<double>(),
+           (const double*)kap, lam, x, dg, nbx, nby, planes);
   SSAMG_LAUNCH_CHECK();
 }
