@@ -1043,7 +1043,7 @@ constexpr int kMaxLevels = 128;
 // round).  Takes the least rounds x (z + 1.5) if it saves a tenth over 8
 // planes.  Measured on 8 x 64^3 (residual 16.4 -> 11.8 us, last relaxation 27.9 ->
 // 22.5 us inside a PCG iteration; 5 uneven parts 14.5 -> 9.7 and 22.6 -> 19.5); beyond
-// four rounds the last one no longer counts.  With off-diagonals per cell the
+// four rounds the last one no longer counts and 8 planes stay.  With off-diagonals per cell the
 // kernels are bound by their seven coefficient streams, not by rounds: 8 planes
 // (2 x 96^3 refined: the solve 2.4 % slower with 10).
 int brick_planes(const Level& L, int per) {
@@ -1058,6 +1058,7 @@ int brick_planes(const Level& L, int per) {
     return (r < 4 ? std::ceil(r) : r + 0.5) * (z + 1.5);
   };
   int best = SSAMG_BRICK_Z;
+  if (bricks(best) >= 4ll * SSAMG_SMS * per) return best;
   for (int z = 4; z <= 16; ++z)
     if (cost(z) < cost(best) && cost(z) < 0.9 * cost(SSAMG_BRICK_Z)) best = z;
   return best;

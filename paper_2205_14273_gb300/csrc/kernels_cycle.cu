@@ -1819,7 +1819,9 @@ bool brick_level(const Level& L) {
 }
 
 // Whether the operator applies of precision T run over bricks: where the tile
-// table says so, else by the rule.  A brick is one block marching 2048 cells,
+// table says so and on large levels (beyond L2 each x is to be read once: 64
+// uneven problems, 72M cells, FP32 residual 403 us over bricks, 722 over tiles),
+// else by the rule.  A brick is one block marching 2048 cells,
 // so a level needs enough of them, well filled; below that the cell tiles
 // spread it further.  Measured (bricks / tiles, us):
 //   FP64 residual, PCG apply, last relaxation: 32^3 (16 bricks) 5.7, 7.8, 9.2 /
@@ -1833,7 +1835,7 @@ bool brick_level(const Level& L) {
 template <class T>
 bool uses_bricks(const Level& L) {
   if (!brick_level(L)) return false;
-  if (L.bricks == 2) return true;
+  if (L.bricks == 2 || L.N >= SSAMG_K7_LARGE) return true;
   return sizeof(T) == 8 ? L.nbblk >= SSAMG_K7_BRICKS_F64 && L.brick_fill >= SSAMG_K7_FILL_F64
                         : L.nbblk >= SSAMG_K7_BRICKS_F32 && L.brick_fill >= SSAMG_K7_FILL_F32;
 }

@@ -47,6 +47,7 @@
 #define SSAMG_SMS 152  // SMs of the GPU (rounds of resident blocks)
 // Fewest bricks of a level, and the least fraction of their cells inside the
 // parts, for the operator applies over bricks (see uses_bricks)
+#define SSAMG_K7_LARGE 5000000  // levels of this many cells always take them
 #define SSAMG_K7_BRICKS_F32 250
 #define SSAMG_K7_FILL_F32 0.6
 #define SSAMG_K7_BRICKS_F64 800
