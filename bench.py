@@ -43,9 +43,9 @@ WORKLOAD = "8 parts x 64^3 (2x2x2 layout), 7-pt anisotropic diffusion, seed 1"
 L2_BYTES = 129 * 2 ** 20
 # FP64 peak of one GB300: 152 SMs x 2 FP64 FMA per clock per SM x 2 flops x 2.07 GHz
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# FP64-pipe instructions per cell of dL/dg (exp(g), then six faces with a
-# division each), counted by ncu on the 128^3 case
-FP64_INSTS_PER_CELL_DG = 15 + 102
+# FP64-pipe instructions per cell of dL/dg: exp(g) (counted by ncu), then three
+# faces of 9, two products a face, kappa^2 and the result (counted in the source)
+FP64_INSTS_PER_CELL_DG = 15 + 39
 
 
 def max_over_ranks(value, ws, device=None):
@@ -794,8 +794,7 @@ def differentiation_workload(S, stream, peak):
             "k_diffusion_exp_gradient": {
                 "us": round(us_dg, 2), "frac_hbm": frac(32 * N, us_dg),
                 # bound by the FP64 pipe: FP64-pipe instructions per cell
-                # counted by ncu (15 in k_exp, 102 in the gradient kernel)
-                # against 2 per SM per clock (152 SMs, 2.07 GHz)
+                # (15 in k_exp, 39 in the gradient kernel) against 2 per SM per clock (152 SMs, 2.07 GHz)
                 "bound": "fp64",
                 "fp64_pipe_insts_per_cell": FP64_INSTS_PER_CELL_DG,
                 "frac_fp64_pipe": round(FP64_INSTS_PER_CELL_DG * N / (us_dg * 1e-6)
