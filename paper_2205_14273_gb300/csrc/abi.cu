@@ -1423,14 +1423,16 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
                                dense || direct, rp);
         const long long smem = a.vec_bytes + a.ro_bytes + a.lo_bytes;
         if (!ok || smem > optin) continue;
+        CTailArgs c{};  // dense: the levels folded into the matrix
+        long long crp[2];
+        if (dense && !(layout(c, tl, Lc, tl, 1, sizeof(double), direct, crp) &&
+                       ctail_columns_prepare(c, optin)))
+          continue;
         const bool can = fp32 ? ctail_prepare<float>(nc, smem) : ctail_prepare<double>(nc, smem);
         if (!can) continue;
         const double* inv = direct ? s->cinv : nullptr;
         if (dense) {
           // the rest of the cycle as a dense matrix
-          CTailArgs c{};
-          long long crp[2];
-          layout(c, tl, Lc, tl, 1, sizeof(double), direct, crp);
           images(c, tl, 1, crp, false, inv);
           double* M = aalloc<double>(s->arena, s->lev[tl].N * s->lev[tl].N);
           launch_ctail_columns(c, M, st);

@@ -749,30 +749,51 @@ void launch_ctail_fill(bool fp32, const std::vector<Level>& lev, int t0, const C
   SSAMG_LAUNCH_CHECK();
 }
 
-void launch_ctail_columns(const CTailArgs& a, double* dense, cudaStream_t st) {
-  const long long vec = (long long)CTAIL_COLS * a.vec_bytes, all = vec + a.lo_bytes;
-  const int staged = all <= SSAMG_CTAIL_STAGE_BYTES;
-  if (staged)
-    SSAMG_CUDA(cudaFuncSetAttribute(k_ctail_columns, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    SSAMG_CTAIL_STAGE_BYTES));
-  k_ctail_columns<<<cdiv(a.lev[0].n, CTAIL_COLS), CT, (size_t)(staged ? all : vec), st>>>(a, staged,
-                                                                                        dense);
-  SSAMG_LAUNCH_CHECK();
-}
-
-// Dynamic shared memory k_ctail<T> is allowed on device dev: at least smem.  The
+// Dynamic shared memory kernel `k` is allowed on device dev: at least smem.  The
 // attribute belongs to the function, not to a launch, so it is never lowered: a
 // solver set up later with a smaller tail must not cut off the launches of one
-// set up before.  (Called with ctail_prepare's lock.)
-template <class T>
-cudaError_t ctail_allow(int dev, long long smem) {
-  static std::map<int, long long> allowed;
-  long long& a = allowed[dev];
+// set up before.
+static cudaError_t allow_smem(const void* k, int dev, long long smem) {
+  static std::mutex mu;
+  static std::map<std::pair<const void*, int>, long long> allowed;
+  std::lock_guard<std::mutex> lock(mu);
+  long long& a = allowed[{k, dev}];
   if (smem <= a) return cudaSuccess;
   const cudaError_t e =
-      cudaFuncSetAttribute(k_ctail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e == cudaSuccess) a = smem;
   return e;
+}
+
+// Shared memory of k_ctail_columns: the vectors of its columns, and the image
+// where both fit SSAMG_CTAIL_STAGE_BYTES.  Without the image it can still be
+// beyond the 48 KB a kernel has by default (levels of more than 1024 cells
+// together, as many small parts leave: 149 parts of 2^3 beside one of 16^3,
+// 1170 cells, 56 KB).
+static long long ctail_columns_smem(const CTailArgs& a, bool& staged) {
+  const long long vec = (long long)CTAIL_COLS * a.vec_bytes, all = vec + a.lo_bytes;
+  staged = all <= SSAMG_CTAIL_STAGE_BYTES;
+  return staged ? all : vec;
+}
+
+bool ctail_columns_prepare(const CTailArgs& a, long long optin) {
+  int dev = 0;
+  bool staged;
+  const long long smem = ctail_columns_smem(a, staged);
+  if (smem > optin) return false;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      allow_smem((const void*)k_ctail_columns, dev, smem) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return true;
+}
+
+void launch_ctail_columns(const CTailArgs& a, double* dense, cudaStream_t st) {
+  bool staged;
+  const long long smem = ctail_columns_smem(a, staged);
+  k_ctail_columns<<<cdiv(a.lev[0].n, CTAIL_COLS), CT, (size_t)smem, st>>>(a, staged, dense);
+  SSAMG_LAUNCH_CHECK();
 }
 
 template <class T>
@@ -790,7 +811,7 @@ bool ctail_prepare(int nc, long long smem) {
   std::lock_guard<std::mutex> lock(mu);
   auto it = known.find(key);
   if (it != known.end()) return it->second;
-  if (ctail_allow<T>(dev, smem) != cudaSuccess) {
+  if (allow_smem((const void*)k_ctail<T>, dev, smem) != cudaSuccess) {
     cudaGetLastError();
     return known[key] = false;
   }

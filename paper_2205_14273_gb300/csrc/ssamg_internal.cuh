@@ -575,6 +575,9 @@ void launch_ctail_fill(bool fp32, const std::vector<Level>& lev, int t0, const C
 // dense (n x n, n = a.lev[0].n): one cycle over the levels of `a` (all local,
 // FP64 common image) applied to every unit vector.
 void launch_ctail_columns(const CTailArgs& a, double* dense, cudaStream_t st);
+// Allows that kernel the shared memory `a` needs; false when it is beyond optin
+// bytes or the device refuses it.
+bool ctail_columns_prepare(const CTailArgs& a, long long optin);
 // Allows the tail kernel nc-CTA clusters and smem bytes of shared memory per
 // CTA; false when the device cannot run such a cluster.
 template <class T>
