@@ -1134,11 +1134,12 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
   {
     // operator-apply shape shared by all parts (see StencilShape)
     bool unchecked = true, all27 = true, all7 = true, all9 = true, all15 = true;
-    bool canon7 = true, canon5 = true;
+    bool canon7 = true, canon5 = true, wide = false;
     static const int c7[7][3] = {{0, 0, 0}, {-1, 0, 0}, {1, 0, 0}, {0, -1, 0},
                                  {0, 1, 0}, {0, 0, -1}, {0, 0, 1}};
     for (const DPart& dp : L.dparts) {
       unchecked = unchecked && dp.allvar && dp.zeroext;
+      wide = wide || (long long)dp.nent * dp.ncell >= (1ll << 31);
       all27 = all27 && dp.canon27;
       all7 = all7 && dp.nent == 7;
       all15 = all15 && dp.nent == 15;
@@ -1149,7 +1150,13 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
         for (int d = 0; d < 3; ++d)
           if (dp.o[e][d] != c7[e][d]) canon7 = canon5 = false;
     }
-    L.shape = !unchecked ? (canon7 ? 5 : canon5 ? 7 : 0) : all27 ? 3 : all7 ? 1 : all9 ? 6 : all15 ? 2 : 4;
+    L.shape = !unchecked ? (canon7 ? 5 : canon5 ? 7 : 0)
+              : wide       ? 8
+              : all27      ? 3
+              : all7       ? 1
+              : all9       ? 6
+              : all15      ? 2
+                           : 4;
     L.kvar = 0;
     for (const DPart& dp : L.dparts)
       L.kvar = std::max(L.kvar, dp.varmask == 0 ? 0 : dp.varmask == 1u ? 1 : 2);

@@ -1,6 +1,8 @@
 // Device helpers shared by the kernel translation units.
 #pragma once
 
+#include <type_traits>
+
 #include "ssamg_internal.cuh"
 
 // Cell-wise launches give each block a tile of P.cpt x SSAMG_BLOCK
@@ -117,7 +119,7 @@ __device__ __forceinline__ float coef_at(const DPart& p, const float* __restrict
 // vector.  The entry count is uniform over a block, so the dispatch below does
 // not diverge.  Fully unrolled variants (7, 15 and 27 entries) issue all loads
 // of a cell together.  Parts whose entries are all per cell (every coarse
-// level) address entry e as a[e * ncell]; the full 27-point stencil in
+// level) address entry e as a[e * ncell] (see SH_UWIDE); the full 27-point stencil in
 // offset-code order derives offsets and bounds from e at compile time.
 template <class T>
 __device__ __forceinline__ T const_of(const DPart& p, int e);
@@ -170,21 +172,23 @@ __device__ __forceinline__ T stencil_fixed(const DPart& p, const T* __restrict__
 
 // Unchecked form: every entry per cell and zero where it leaves the box, and x
 // readable (finite) one plane beyond each end of the level vector, so every
-// cell takes the same path with no bounds tests.
-template <int K, class T>
+// cell takes the same path with no bounds tests.  I: the type of an entry's offset
+// e * ncell, see SH_UWIDE.
+template <int K, class I = int, class T>
 __device__ __forceinline__ T stencil_unchecked(const DPart& p, const T* __restrict__ a,
                                                const T* __restrict__ xc) {
-  const int s = p.ncell;
+  const I s = p.ncell;
   T acc = (T)0;
 #pragma unroll
   for (int e = 0; e < K; ++e) acc = fma(a[e * s], xc[p.disp[e]], acc);
   return acc;
 }
 
-template <class T>
+template <class I = int, class T>
 __device__ __forceinline__ T stencil27_unchecked(const DPart& p, const T* __restrict__ a,
                                                  const T* __restrict__ xc) {
-  const int nx = p.n[0], nxy = p.n[0] * p.n[1], s = p.ncell;
+  const int nx = p.n[0], nxy = p.n[0] * p.n[1];
+  const I s = p.ncell;
   T acc = (T)0;
 #pragma unroll
   for (int e = 0; e < 27; ++e) {
@@ -240,8 +244,14 @@ __device__ __forceinline__ bool is_interior(const DPart& p, int i, int j, int k)
 // checked 5-point stencil on level 0.  Four 511 x 509 parts, FP64: 9-point
 // residual of 520,000 cells 37.6 -> 18.9 us, 5-point 19.2 -> 16.4 us, against the
 // general loops.)
+// UWIDE is UGEN for levels with a part whose entries pass 2^31 elements together
+// (27 entries from 79.6M cells, 15 from 143.2M): entry offsets of 64 bits.  The
+// other unchecked shapes keep 32: with 64 the isolated kernels are as fast, but
+// a cycle of 8 x 64^3 FP32 (15 entries) takes 291 instead of 287 us and a refined
+// 2 x 96^3 solve 30.9 instead of 30.4 ms.
 enum StencilShape {
-  SH_CHECKED = 0, SH_U7 = 1, SH_U15 = 2, SH_C27 = 3, SH_UGEN = 4, SH_K7 = 5, SH_U9 = 6, SH_K5 = 7
+  SH_CHECKED = 0, SH_U7 = 1, SH_U15 = 2, SH_C27 = 3, SH_UGEN = 4, SH_K7 = 5, SH_U9 = 6, SH_K5 = 7,
+  SH_UWIDE = 8
 };
 
 // Checked 7-point stencil (K = 5: 5-point, 2-D) in the canonical entry order
@@ -334,16 +344,18 @@ __device__ __forceinline__ T stencil_sh(const DPart& p, const T* __restrict__ co
     return stencil7_canon_checked<5>(p, coef, xc, c, i, j, k);
   } else if constexpr (SH == SH_U9) {
     return stencil_unchecked<9>(p, coef + p.coef[0] + c, xc);
-  } else if constexpr (SH == SH_UGEN) {
+  } else if constexpr (SH == SH_UGEN || SH == SH_UWIDE) {
     // parts of one level with different stencils (e.g. semicoarsened in
     // different directions): the unrolled form of each part's size, chosen
     // per part (uniform over a block), so that every entry's loads are in
     // flight together; the same entry order as a plain loop
     const T* a = coef + p.coef[0] + c;
-    if (p.canon27) return stencil27_unchecked(p, a, xc);
-    if (p.nent == 15) return stencil_unchecked<15>(p, a, xc);
-    if (p.nent == 7) return stencil_unchecked<7>(p, a, xc);
-    const int s = p.ncell, n = p.nent;
+    using I = std::conditional_t<SH == SH_UWIDE, long long, int>;
+    if (p.canon27) return stencil27_unchecked<I>(p, a, xc);
+    if (p.nent == 15) return stencil_unchecked<15, I>(p, a, xc);
+    if (p.nent == 7) return stencil_unchecked<7, I>(p, a, xc);
+    const int n = p.nent;
+    const I s = p.ncell;
     T acc = (T)0;
 #pragma unroll
     for (int e = 0; e < SSAMG_MAXE; ++e)
@@ -405,7 +417,7 @@ __device__ __forceinline__ void stencil27_unchecked_r(const DPart& p, const T* _
   }
 }
 
-// Shapes with a several-right-hand-side form: every entry per cell.
+// Shapes with a several-right-hand-side form: every entry per cell, offsets of 32 bits.
 __host__ __device__ constexpr bool shape_has_rhs_form(int sh) {
   return sh == SH_U7 || sh == SH_U9 || sh == SH_U15 || sh == SH_C27 || sh == SH_UGEN;
 }

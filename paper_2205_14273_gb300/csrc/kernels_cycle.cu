@@ -1194,7 +1194,7 @@ __global__ void k_cast_f2d(const float* in, double* out, int n) {
 
 // y = A x for a caller's x, which has no guard cells: entries that leave the
 // box read the cell itself and are multiplied by zero.  K: 27 for the 27
-// entries in offset-code order, else the level's number of entries, unrolled
+// entries in offset-code order (32-bit entry offsets: SH_C27 alone), else the level's number of entries, unrolled
 // (every load of a cell in flight together), 0 for any.  8 parts of 64^3 (7
 // entries, per-cell diagonal) run over bricks:
 // 52.9 -> 39.1 us with the U x launch before it, of 25 us for the FP64 pipe (7
@@ -1890,6 +1890,7 @@ void launch_relax0_u(const Level& L, const T* b, T* x, cudaStream_t st) {
     case SH_K7: { constexpr int SHV = SH_K7; KCALL; } break;   \
     case SH_U9: { constexpr int SHV = SH_U9; KCALL; } break;   \
     case SH_K5: { constexpr int SHV = SH_K5; KCALL; } break;   \
+    case SH_UWIDE: { constexpr int SHV = SH_UWIDE; KCALL; } break; \
     default: { constexpr int SHV = SH_CHECKED; KCALL; } break; \
   }
 
