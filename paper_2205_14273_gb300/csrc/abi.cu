@@ -1423,6 +1423,10 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
         const int tl = std::max(small, t0);
         if (form && tl >= Lc) continue;
         const bool dense = form && !fp32;
+        // (independent problems without the coarsest inverse, which couples
+        // them already: the matrix's zeros between them times one problem's NaN
+        // or infinity would spoil the others)
+        if (dense && s->nprob > 1 && !direct) continue;
         CTailArgs a{};
         a.dense = dense;
         long long rp[2];
