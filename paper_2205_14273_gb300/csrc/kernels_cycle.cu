@@ -1625,7 +1625,12 @@ __device__ __forceinline__ double dg_cell(const DPart& sp, const double* kap, co
 // A thread per cell: boxes below SSAMG_DG_CELLS cells, whose few blocks leave the
 // FP64 pipe idle, so that the shared-face form's barriers cost more than its
 // instructions save (passes one after another: 32^3 12.8 us, host-bound, vs 23.6;
-// 40^3 43 vs 27 us).
+// 40^3 43 vs 27 us), and boxes that fill less than SSAMG_DG_FILL of the other
+// form's columns, whose threads take the instructions of cells that are not there
+// (cells' form / shared faces, us; nx x ny x nz: 64 x 1 x 4000, fill 0.12, 49 / 148;
+// 33 x 9 x 4000, 0.29, 268 / 345; 12 x 100 x 200, 0.36, 63 / 76; 33 x 33 x 400,
+// 0.43, 105 / 110; 34^3, 0.45, 22 / 24; 16 x 100 x 200, 0.48, 80 / 77; 65 x 65 x 200,
+// 0.61, 189 / 151).
 __global__ void __launch_bounds__(NT) k_diffusion_exp_cells(LevelView<double> L, const double* kap,
                                                             const double* lam, const double* x,
                                                             double* dg) {
@@ -2266,16 +2271,16 @@ void launch_diffusion_exp_gradient(const Level& L, const double* g, const double
   const int n = (int)L.parts[0].ncell;
   launch_k(k_exp, cdiv(n, NT), NT, 0, st, n, g, kap);
   SSAMG_LAUNCH_CHECK();
-  if (n < SSAMG_DG_CELLS) {
+  const int* e = L.parts[0].n;
+  const int nbx = cdiv(e[0], GX), nby = cdiv(e[1], GY);
+  const long long cols = (long long)nbx * nby;
+  if (n < SSAMG_DG_CELLS || n < SSAMG_DG_FILL * (double)(cols * (GX * GY) * e[2])) {
     launch_k(k_diffusion_exp_cells, cdiv(n, NT), NT, 0, st, L.view<double>(), (const double*)kap, lam,
              x, dg);
     SSAMG_LAUNCH_CHECK();
     return;
   }
-  const int* e = L.parts[0].n;
-  const int nbx = cdiv(e[0], GX), nby = cdiv(e[1], GY);
   // as many planes as leave four blocks an SM
-  const long long cols = (long long)nbx * nby;
   const int planes = (int)std::max(1ll, std::min((long long)GZ, cols * e[2] / (4 * SSAMG_SMS)));
   launch_k(k_diffusion_exp_gradient, (int)(cols * cdiv(e[2], planes)), NT, 0, st, L.view<double>(),
            (const double*)kap, lam, x, dg, nbx, nby, planes);

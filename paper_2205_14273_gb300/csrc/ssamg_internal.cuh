@@ -53,6 +53,7 @@
 #define SSAMG_K7_BRICKS_F64 800
 #define SSAMG_K7_FILL_F64 0.85
 #define SSAMG_DG_CELLS (152 * 256)  // smaller boxes (a block an SM) take dL/dg with a thread per cell
+#define SSAMG_DG_FILL 0.47  // and boxes that fill less of the shared-face form's 32 x 8 columns
 #define SSAMG_RP_BRICKS 152  // fewest bricks for the restriction / prolongation brick forms
 #define SSAMG_RP_FILL 0.8    // and the least fraction of their brick cells inside the parts
 #define SSAMG_TPR 4       // fewest lanes per U row in row jobs
