@@ -294,12 +294,14 @@ struct ssamg_matrix_s {
 
 // The instantiated solve graphs, each with the state its launches were captured
 // from (every pointer, count and form they take, see graph_signature): a
-// set-up that leaves all of it as it was (a new operator of the same shape on
-// the same solver walks the same arena) keeps the graph, whose capture and
-// instantiation take 0.2 ms (45 nodes) to 1 ms (four right-hand sides).
+// set-up that leaves all of it as it was keeps the graph, whose capture and
+// instantiation take 0.2 ms (45 nodes) to 1 ms (four right-hand sides).  The
+// solver's arrays come from the same walk of its arena when the hierarchy has the
+// same shape; level 0's belong to the matrix, so the graph stays when the same
+// matrix is set up again, and over a new assembly of it when the allocator returns
+// the same blocks (without couplings it does as a rule, with them seldom).
 struct GraphSet {
   cudaGraphExec_t pcg = nullptr;
-  cudaGraphExec_t vcycle = nullptr;
   cudaGraphExec_t rounds = nullptr;  // several right-hand sides in one graph
   std::vector<char> pcg_sig, rounds_sig;
   static void drop(cudaGraphExec_t& g) {
@@ -308,7 +310,6 @@ struct GraphSet {
   }
   void reset() {
     drop(pcg);
-    drop(vcycle);
     drop(rounds);
   }
 };
@@ -1161,8 +1162,7 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
     for (const DPart& dp : L.dparts)
       L.kvar = std::max(L.kvar, dp.varmask == 0 ? 0 : dp.varmask == 1u ? 1 : 2);
   }
-  // (resident blocks an SM: the launch bounds of the kernels)
-  const int per[2] = {6, 5};
+  const int per[2] = {SSAMG_BRICK_RESIDENT_F32, SSAMG_BRICK_RESIDENT_FINAL32};
   for (int q = 0; q < 2; ++q) {
     L.bf[q].z = L.kvar == 2 ? SSAMG_BRICK_Z : brick_planes(L, per[q]);
     t.kb[q].assign(np + 1, 0);
@@ -1323,9 +1323,9 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
       v.S = v.local ? v.n : slice;
       if (v.S >= (1 << SSAMG_CTAIL_LOCAL_BITS)) return false;
       // lanes per row: as many as leave every row of the slice a group in one
-      // pass (of a local level too, so that its sums keep the cluster's order)
-      // (FP64: few lanes, the pipe takes 16 cycles for each add of a lane tree;
-      // the dense matrix's columns have half a block each)
+      // pass (FP64: few lanes, the pipe takes 16 cycles for each add of a lane
+      // tree; the dense matrix's columns have half a block each; FP32 local
+      // levels choose their own, see ctail_apply_rows)
       const int most = w == 8 ? SSAMG_CTAIL_TPR_F64 : 32;
       const int threads = nc > 1 ? SSAMG_CTAIL_THREADS : SSAMG_CTAIL_THREADS / 2;
       v.tpr = 1;
@@ -1416,7 +1416,8 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
   int small = lt;
   while (small < Lc && s->lev[small].N > (fp32 ? SSAMG_CTAIL_LOCAL_CELLS : SSAMG_CTAIL_DENSE_CELLS)) ++small;
   for (int nc : {SSAMG_CTAIL_MAX_CTAS, 8}) {
-    for (int t0 = lt; t0 < Lc; ++t0) {
+    bool refused = false;  // by the device, in the form with less shared memory too: fewer CTAs
+    for (int t0 = lt; t0 < Lc && !refused; ++t0) {
       if (Lc - t0 + 1 > SSAMG_CTAIL_MAX_LEVELS) continue;
       for (int form = small < Lc ? 1 : 0; form >= 0; --form) {
         // form 1: levels from max(small, t0) on local (FP32) or dense (FP64)
@@ -1439,8 +1440,8 @@ void build_ctail(ssamg_solver s, cudaStream_t st) {
         if (dense && !(layout(c, tl, Lc, tl, 1, sizeof(double), direct, crp) &&
                        ctail_columns_prepare(c, optin)))
           continue;
-        const bool can = fp32 ? ctail_prepare<float>(nc, smem) : ctail_prepare<double>(nc, smem);
-        if (!can) continue;
+        refused = !(fp32 ? ctail_prepare<float>(nc, smem) : ctail_prepare<double>(nc, smem));
+        if (refused) continue;
         const double* inv = direct ? s->cinv : nullptr;
         if (dense) {
           // the rest of the cycle as a dense matrix

@@ -116,59 +116,17 @@ __device__ __forceinline__ float coef_at(const DPart& p, const float* __restrict
 }
 
 // (S x)(c) for local cell c = (i, j, k) of part p; x points at the level
-// vector.  The entry count is uniform over a block, so the dispatch below does
+// vector.  The entry count is uniform over a block, so a choice by it does
 // not diverge.  Fully unrolled variants (7, 15 and 27 entries) issue all loads
 // of a cell together.  Parts whose entries are all per cell (every coarse
-// level) address entry e as a[e * ncell] (see SH_UWIDE); the full 27-point stencil in
-// offset-code order derives offsets and bounds from e at compile time.
+// level) address entry e as a[e * ncell] (see SH_UWIDE); the full 27-point
+// stencil in offset-code order derives offsets and bounds from e at compile time.
 template <class T>
 __device__ __forceinline__ T const_of(const DPart& p, int e);
 template <>
 __device__ __forceinline__ double const_of<double>(const DPart& p, int e) { return p.cval[e]; }
 template <>
 __device__ __forceinline__ float const_of<float>(const DPart& p, int e) { return p.cval32[e]; }
-
-template <class T>
-__device__ __forceinline__ T stencil27_canon(const DPart& p, const T* __restrict__ a,
-                                             const T* __restrict__ xc, int i, int j, int k,
-                                             bool interior) {
-  const int nx = p.n[0], nxy = p.n[0] * p.n[1], s = p.ncell;
-  const bool xm = i > 0, xp = i < p.n[0] - 1, ym = j > 0, yp = j < p.n[1] - 1, zm = k > 0,
-             zp = k < p.n[2] - 1;
-  T acc = (T)0;
-#pragma unroll
-  for (int e = 0; e < 27; ++e) {
-    const int dx = e % 3 - 1, dy = (e / 3) % 3 - 1, dz = e / 9 - 1;
-    const bool ok = interior || ((dx == 0 || (dx < 0 ? xm : xp)) && (dy == 0 || (dy < 0 ? ym : yp)) &&
-                                 (dz == 0 || (dz < 0 ? zm : zp)));
-    if (ok) acc = fma(a[e * s], xc[dx + dy * nx + dz * nxy], acc);
-  }
-  return acc;
-}
-
-template <int K, class T>
-__device__ __forceinline__ T stencil_fixed(const DPart& p, const T* __restrict__ coef,
-                                           const T* __restrict__ xc, int c, int i, int j, int k,
-                                           bool interior) {
-  T acc = (T)0;
-  if (p.allvar) {
-    const T* a = coef + p.coef[0] + c;
-    const int s = p.ncell;
-#pragma unroll
-    for (int e = 0; e < K; ++e)
-      if (interior || inside(p, i + p.o[e][0], j + p.o[e][1], k + p.o[e][2]))
-        acc = fma(a[e * s], xc[p.disp[e]], acc);
-  } else {
-    const unsigned vm = p.varmask;
-#pragma unroll
-    for (int e = 0; e < K; ++e)
-      if (interior || inside(p, i + p.o[e][0], j + p.o[e][1], k + p.o[e][2])) {
-        const T ae = ((vm >> e) & 1u) ? coef[p.coef[e] + c] : const_of<T>(p, e);
-        acc = fma(ae, xc[p.disp[e]], acc);
-      }
-  }
-  return acc;
-}
 
 // Unchecked form: every entry per cell and zero where it leaves the box, and x
 // readable (finite) one plane beyond each end of the level vector, so every
@@ -195,36 +153,6 @@ __device__ __forceinline__ T stencil27_unchecked(const DPart& p, const T* __rest
     const int dx = e % 3 - 1, dy = (e / 3) % 3 - 1, dz = e / 9 - 1;
     acc = fma(a[e * s], xc[dx + dy * nx + dz * nxy], acc);
   }
-  return acc;
-}
-
-template <class T>
-__device__ __forceinline__ T stencil_apply(const DPart& p, const T* __restrict__ coef,
-                                           const T* __restrict__ x, int c, int i, int j, int k,
-                                           bool interior, bool padded) {
-  const T* xc = x + p.off + c;
-  if (p.allvar && p.zeroext && padded) {
-    const T* a = coef + p.coef[0] + c;
-    if (p.canon27) return stencil27_unchecked(p, a, xc);
-    switch (p.nent) {
-      case 7: return stencil_unchecked<7>(p, a, xc);
-      case 15: return stencil_unchecked<15>(p, a, xc);
-      case 27: return stencil_unchecked<27>(p, a, xc);
-      default: break;
-    }
-  }
-  if (p.canon27 && p.allvar) return stencil27_canon(p, coef + p.coef[0] + c, xc, i, j, k, interior);
-  switch (p.nent) {
-    case 7: return stencil_fixed<7>(p, coef, xc, c, i, j, k, interior);
-    case 15: return stencil_fixed<15>(p, coef, xc, c, i, j, k, interior);
-    case 27: return stencil_fixed<27>(p, coef, xc, c, i, j, k, interior);
-    default: break;
-  }
-  T acc = (T)0;
-#pragma unroll 4
-  for (int e = 0; e < p.nent; ++e)
-    if (interior || inside(p, i + p.o[e][0], j + p.o[e][1], k + p.o[e][2]))
-      acc = fma(coef_at(p, coef, e, c), xc[p.disp[e]], acc);
   return acc;
 }
 
@@ -472,31 +400,6 @@ __device__ __forceinline__ void apply_A_sh_r(const LevelView<T>& L, const DPart&
 #pragma unroll
     for (int q = 0; q < R; ++q) acc[q] += L.uy[p.off + c + q * vs];
   }
-}
-
-// (U x)(g) for global cell g (0 when g has no U row).
-template <class T>
-__device__ __forceinline__ T u_apply(const LevelView<T>& L, const T* __restrict__ x, int g) {
-  int r = __ldg(L.u_map + g);
-  T acc = (T)0;
-  if (r >= 0) {
-    int q1 = __ldg(L.u_ptr + r + 1);
-    for (int q = __ldg(L.u_ptr + r); q < q1; ++q) acc = fma(L.u_val[q], x[__ldg(L.u_col + q)], acc);
-  }
-  return acc;
-}
-
-
-// (A x)(c) = (S x)(c) + (U x)(c); the U part comes from L.uy, which a row
-// job filled for this same x (only face cells can have couplings unless
-// has_u is 2).
-template <class T>
-__device__ __forceinline__ T apply_A(const LevelView<T>& L, const DPart& p, const T* __restrict__ x,
-                                     int c, int i, int j, int k, bool padded = true) {
-  bool interior = is_interior(p, i, j, k);
-  T acc = stencil_apply(p, L.coef, x, c, i, j, k, interior, padded);
-  if (p.has_u > 1 || (p.has_u && !interior)) acc += L.uy[p.off + c];
-  return acc;
 }
 
 // Sum of one U row: the L.tpr lanes l4 of a row group compute

@@ -313,7 +313,7 @@ F pick_km(int km, F f0, F f1, F f2) {
 // as many as fit without register spills.
 template <class T, int KM>
 constexpr int brick_min_blocks() {
-  return sizeof(T) == 8 ? (KM == 2 ? 4 : 5) : (KM == 2 ? 5 : 6);
+  return sizeof(T) == 8 ? (KM == 2 ? 4 : 5) : (KM == 2 ? 5 : SSAMG_BRICK_RESIDENT_F32);
 }
 
 template <class T>
@@ -406,7 +406,7 @@ __global__ void __launch_bounds__(NT, brick_min_blocks<T, KM>()) k7b_relax(Level
 }
 
 template <class T, int KM>
-__global__ void __launch_bounds__(NT, sizeof(T) == 4 && KM < 2 ? 5 : 4) k7b_relax_final(LevelView<T> L, BrickForm f, const T* x, const T* b,
+__global__ void __launch_bounds__(NT, sizeof(T) == 4 && KM < 2 ? SSAMG_BRICK_RESIDENT_FINAL32 : 4) k7b_relax_final(LevelView<T> L, BrickForm f, const T* x, const T* b,
                                                       double* z, const double* rpcg, int flex,
                                                       double* partial) {
   pdl_trigger();

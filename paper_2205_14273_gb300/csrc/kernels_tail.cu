@@ -22,7 +22,7 @@
 // four barriers and remote round trips as the others, ~3.8 us (FP32) and
 // ~4.7 us (FP64) each, with nothing to spread.  In FP32 every CTA holds them
 // whole and runs them for itself: block barriers and its own shared memory,
-// each row summed as the cluster would.  In FP64 an SM's two multiply-adds per
+// each row summed as a cluster of 16 would.  In FP64 an SM's two multiply-adds per
 // clock forbid that (256 rows x 30 entries are 2 us an apply); there the rest
 // of the cycle from the first such level down, a linear map of its right-hand
 // side, is formed at setup as a dense matrix (one block per column runs that
@@ -317,9 +317,10 @@ __device__ __forceinline__ void ctail_apply(cg::cluster_group& cl, char* sm, int
 
 // Sum of entries [q, q1) of a local level's row by G neighbouring lanes, lane
 // h of them holding the partial sums of ctail_apply's lanes h, h + G, ... in
-// registers: its tree (a level of at most SSAMG_CTAIL_LOCAL_CELLS cells has 32
-// lanes a row there), within a lane as far as it goes, so the result is the
-// same bit for bit with log2 G shuffles.  All lanes of the warp call.
+// registers: its tree, within a lane as far as it goes, with log2 G shuffles.
+// With 16 CTAs a level of at most SSAMG_CTAIL_LOCAL_CELLS cells has 32 lanes a row
+// there and the result is the same bit for bit (with 8 CTAs and more than 128
+// cells it has 16, another order).  All lanes of the warp call.
 template <int G, class T>
 __device__ __forceinline__ T ctail_row_sum(const T* x, const unsigned short* col, const T* val,
                                            int q, int q1) {

@@ -45,6 +45,10 @@
 #define SSAMG_BRICK_Y 8
 #define SSAMG_BRICK_Z 8
 #define SSAMG_SMS 152  // SMs of the GPU (rounds of resident blocks)
+// Resident blocks an SM of the FP32 brick applies without off-diagonals per
+// cell: launch bounds of the kernels, and rounds in the choice of their planes
+#define SSAMG_BRICK_RESIDENT_F32 6  // residual, relaxation
+#define SSAMG_BRICK_RESIDENT_FINAL32 5  // last relaxation
 // Fewest bricks of a level, and the least fraction of their cells inside the
 // parts, for the operator applies over bricks (see uses_bricks)
 #define SSAMG_K7_LARGE 5000000  // levels of this many cells always take them
@@ -251,7 +255,8 @@ struct LevelView {
 struct CTailLevel {
   int n, S;                  // cells, rows per CTA slice
   int local;                 // 1: whole in every CTA
-  int tpr;                   // lanes per CSR row in the operator applies (power of two <= 32)
+  int tpr;                   // lanes per CSR row in the operator applies (power of two <= 32; not of
+                             // FP32 local levels)
   int o_x, o_b, o_r;         // the level's vectors
   int o_rowptr, o_col, o_val, o_dinv;  // CSR of A = S + U (local row pointers), omega M^-1
   int o_pcol, o_pval;        // P's row of each fine cell (2 per row), to the next level
@@ -266,7 +271,7 @@ struct CTailArgs {
   int nt;                    // tail levels in this form (>= 1)
   int jl;                    // first local level (nt: none)
   int direct;                // 1: last level by its explicit matrix, 0: one relaxation sweep
-  int dense;                 // 1: that matrix is the rest of the cycle (a warp per row)
+  int dense;                 // 1: that matrix is the rest of the cycle (eight lanes per row)
   int o_sb;                  // dense: the last level's b gathered (FP64)
   int nL;                    // cells of the last level
   CTailLevel lev[SSAMG_CTAIL_MAX_LEVELS];
