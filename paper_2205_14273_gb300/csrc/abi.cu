@@ -1056,7 +1056,7 @@ int brick_planes(const Level& L, int per) {
   };
   auto cost = [&](int z) {
     const double r = (double)bricks(z) / (SSAMG_SMS * per);
-    return (r < 4 ? std::ceil(r) : r + 0.5) * (z + 1.5);
+    return (r < 4 ? std::ceil(r) : r + 0.5) * (z + SSAMG_BRICK_LEAD);
   };
   int best = SSAMG_BRICK_Z;
   if (bricks(best) >= 4ll * SSAMG_SMS * per) return best;
@@ -1110,6 +1110,15 @@ void level_tables(ssamg_solver s, Level& L, const Level* next, LevelTables& t) {
   L.brick_fill = L.nbblk ? (double)ntot / ((double)L.nbblk * SSAMG_BRICK_X * SSAMG_BRICK_Y *
                                            SSAMG_BRICK_Z)
                          : 0.0;
+  {
+    // the same by the time the bricks take: their planes and SSAMG_BRICK_LEAD more
+    double planes = 0.0;
+    for (const PartH& h : L.parts)
+      planes += (double)(cdivll(h.n[0], SSAMG_BRICK_X) * cdivll(h.n[1], SSAMG_BRICK_Y)) *
+                (h.n[2] + SSAMG_BRICK_LEAD * cdivll(h.n[2], SSAMG_BRICK_Z));
+    L.brick_march = ntot * (1.0 + SSAMG_BRICK_LEAD / SSAMG_BRICK_Z) /
+                    (planes * SSAMG_BRICK_X * SSAMG_BRICK_Y);
+  }
   L.hbblk = bblk;
   L.hblk = blk;
   for (int p = 0; p < np; ++p) {
@@ -2207,7 +2216,7 @@ std::vector<char> graph_signature(ssamg_solver s) {
         L.dinv32, L.Pw, L.Pe, L.Pw32, L.Pe32, L.u_map, L.u_ptr, L.u_rows, L.u_col, L.u_val,
         L.u_val32, L.u_bits, L.u_pj, L.u_pw, L.u_pw32, L.u_rj, L.u_rw, L.u_rw32, L.uy64, L.uy32);
     put(L.nr, L.nnz, L.u_rb, L.nublk, L.tpr, L.nblk, L.nfblk, L.nbblk, L.cpt, L.bricks, L.brick_fill,
-        L.kvar, L.shape, L.guard, L.x, L.b, L.r, L.t);
+        L.brick_march, L.kvar, L.shape, L.guard, L.x, L.b, L.r, L.t);
     for (const BrickForm& f : L.bf) put(f.blk, f.z, f.n);
   }
   put(s->nprob, s->nL, s->chol, s->cinv, s->tail_lt, s->tail_dev, s->tail_blocks, s->tail_bar,

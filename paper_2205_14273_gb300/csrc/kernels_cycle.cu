@@ -1828,21 +1828,27 @@ bool brick_level(const Level& L) {
 // uneven problems, 72M cells, FP32 residual 403 us over bricks, 722 over tiles),
 // else by the rule.  A brick is one block marching 2048 cells,
 // so a level needs enough of them, well filled; below that the cell tiles
-// spread it further.  Measured (bricks / tiles, us):
+// spread it further.  The fill is by the bricks' time (brick_march): the bricks
+// of parts of a few planes end early, so that many tiny parts beside a large one
+// do not take it off its bricks (FP32 solve over bricks / tiles: 200 parts of 2^3
+// and one of 64^3, 0.64 by time but 0.39 by cells, 1.81 / 1.89 ms; 500 and 96^3,
+// 0.70, 3.72 / 3.81; 300 and 128^3, 0.90, 4.49 / 4.71; 60 parts of 64 x 64 x 4,
+// 0.86, 2.10 / 2.17; 40 of 100 x 100 x 3, 0.59, 2.59 / 2.47).  Measured (bricks /
+// tiles, us; bricks and fill):
 //   FP64 residual, PCG apply, last relaxation: 32^3 (16 bricks) 5.7, 7.8, 9.2 /
 //     2.7, 5.0, 4.6; 8 x 48^3 (576, 0.75 full) 25, 27, 30 / 16, 26, 26; 100^3
-//     (676, 0.72) 22, 29, 44 / 17, 20, 26; 8 x 56^3 (784, 0.88) 30, 37, 43 / 27, 37,
+//     (676, 0.75) 22, 29, 44 / 17, 20, 26; 8 x 56^3 (784, 0.88) 30, 37, 43 / 27, 37,
 //     42; 8 x 72^3 (1944, 0.75) 67, 73, 92 / 55, 64, 78; 2 x 96^3 (864, full) 37, 44,
 //     58 / 35, 47, 51; 8 x 64^3 (1024, full) 37, 42, 52 / 37, 48, 60
-//   FP32 residual, last relaxation: 32^3 3.0, 5.8 / 1.5, 3.3; 8 x 33^3 (400, 0.35)
+//   FP32 residual, last relaxation: 32^3 3.0, 5.8 / 1.5, 3.3; 8 x 33^3 (400, 0.41)
 //     6.6, 12.6 / 3.9, 7.8; 80^3 (300, 0.83) 4.0, 11.7 / 4.2, 7.3; 8 x 48^3 7.6, 13.0
 //     / 6.8, 13.3; 100^3 5.9, 12.9 / 6.7, 12.7; 8 x 64^3 9.9, 24.5 / 14.2, 35.6
 template <class T>
 bool uses_bricks(const Level& L) {
   if (!brick_level(L)) return false;
   if (L.bricks == 2 || L.N >= SSAMG_K7_LARGE) return true;
-  return sizeof(T) == 8 ? L.nbblk >= SSAMG_K7_BRICKS_F64 && L.brick_fill >= SSAMG_K7_FILL_F64
-                        : L.nbblk >= SSAMG_K7_BRICKS_F32 && L.brick_fill >= SSAMG_K7_FILL_F32;
+  return sizeof(T) == 8 ? L.nbblk >= SSAMG_K7_BRICKS_F64 && L.brick_march >= SSAMG_K7_FILL_F64
+                        : L.nbblk >= SSAMG_K7_BRICKS_F32 && L.brick_march >= SSAMG_K7_FILL_F32;
 }
 template bool uses_bricks<float>(const Level&);
 template bool uses_bricks<double>(const Level&);

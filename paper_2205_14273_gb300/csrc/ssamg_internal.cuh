@@ -44,13 +44,14 @@
 #define SSAMG_BRICK_X 32
 #define SSAMG_BRICK_Y 8
 #define SSAMG_BRICK_Z 8
+#define SSAMG_BRICK_LEAD 1.5  // planes of time a brick takes beside the ones it marches
 #define SSAMG_SMS 152  // SMs of the GPU (rounds of resident blocks)
 // Resident blocks an SM of the FP32 brick applies without off-diagonals per
 // cell: launch bounds of the kernels, and rounds in the choice of their planes
 #define SSAMG_BRICK_RESIDENT_F32 6  // residual, relaxation
 #define SSAMG_BRICK_RESIDENT_FINAL32 5  // last relaxation
-// Fewest bricks of a level, and the least fraction of their cells inside the
-// parts, for the operator applies over bricks (see uses_bricks)
+// Fewest bricks of a level, and the least of Level::brick_march, for the operator
+// applies over bricks (see uses_bricks)
 #define SSAMG_K7_LARGE 5000000  // levels of this many cells always take them
 #define SSAMG_K7_BRICKS_F32 250
 #define SSAMG_K7_FILL_F32 0.6
@@ -347,6 +348,7 @@ struct Level {
   BrickForm bf[BF_FORMS] = {};  // bricks of the operator applies (levels that may run over them)
   int bricks = 1; // operator applies over bricks: 0 never, 1 by the rule, 2 the table wants them
   double brick_fill = 0.0;  // cells / (bricks x brick cells): how full the level's bricks are
+  double brick_march = 0.0; // the same by their time (1: full bricks of SSAMG_BRICK_Z planes)
   int kvar = 2;   // per-cell stencil entries: 0 none, 1 only diagonals, 2 others too
   int shape = 0;  // StencilShape of the level's operator apply
   std::vector<int> hblk;  // host copy of the block starts of cell-wise launches
