@@ -1193,15 +1193,17 @@ __global__ void k_cast_f2d(const float* in, double* out, int n) {
 }
 
 // y = A x for a caller's x, which has no guard cells: entries that leave the
-// box read the cell itself and are multiplied by zero.  K: 27 for the 27
-// entries in offset-code order (32-bit entry offsets: SH_C27 alone), else the level's number of entries, unrolled
-// (every load of a cell in flight together), 0 for any.  8 parts of 64^3 (7
-// entries, per-cell diagonal) run over bricks:
-// 52.9 -> 39.1 us with the U x launch before it, of 25 us for the FP64 pipe (7
+// box read the cell itself and are multiplied by zero.  A loop over the entries,
+// four loads ahead, at full occupancy: unrolled by the level's number of entries
+// the kernel lost to it (loop / unrolled, us: 5 entries, 4M cells 41 / 47; 7 per
+// cell, 2.1M 50 / 59; 9, 2M 49 / 99; 15, 1.1M 45 / 76).  C27: the 27 entries in
+// offset-code order unrolled (32-bit entry offsets: SH_C27 alone), for levels
+// without couplings (4.1M cells 227 / 220, 0.9M 64 / 62; with couplings 3.1M 180 /
+// 189).  8 parts of 64^3 (7 entries, per-cell diagonal) run over bricks: 52.9 ->
+// 39.1 us with the U x launch before it, of 25 us for the FP64 pipe (7
 // multiply-adds a cell).
-template <int K>
-__global__ void __launch_bounds__(NT, K == 15 ? 2 : 4)
-    k_matvec(LevelView<double> L, const double* x, double* y) {
+template <bool C27>
+__global__ void __launch_bounds__(NT, 4) k_matvec(LevelView<double> L, const double* x, double* y) {
   pdl_trigger();
   __shared__ DPart sp;
   block_part(L.blk, L.parts, L.np, sp);
@@ -1212,10 +1214,8 @@ __global__ void __launch_bounds__(NT, K == 15 ? 2 : 4)
     cell_coords(sp, c, i, j, k);
     const double* xc = x + sp.off + c;
     double acc;
-    if constexpr (K == 27)
+    if constexpr (C27)
       acc = stencil27_checked(sp, L.coef + sp.coef[0] + c, xc, i, j, k);
-    else if constexpr (K > 0)
-      acc = stencil_checked_fixed<K>(sp, L.coef, xc, c, i, j, k);
     else
       acc = stencil_checked_loop(sp, L.coef, xc, c, i, j, k);
     if (sp.has_u > 1 || (sp.has_u && !is_interior(sp, i, j, k))) acc += L.uy[sp.off + c];
@@ -2173,16 +2173,8 @@ void launch_matvec(const Level& L, const double* x, double* y, cudaStream_t st) 
     launch_k(pick_km(L.kvar, k7b_matvec<0>, k7b_matvec<1>, k7b_matvec<2>), L.bf[BF_64].n, NT, 0, st,
              L.view<double>(), L.bf[BF_64], x, y);
   } else {
-    int ne = L.parts[0].nent;
-    for (const PartH& h : L.parts)
-      if (h.nent != ne) ne = 0;
-    auto kern = L.shape == SH_C27 ? k_matvec<27>
-                : ne == 15        ? k_matvec<15>
-                : ne == 9         ? k_matvec<9>
-                : ne == 7         ? k_matvec<7>
-                : ne == 5         ? k_matvec<5>
-                                  : k_matvec<0>;
-    launch_k(kern, L.nblk, NT, 0, st, L.view<double>(), x, y);
+    launch_k(L.shape == SH_C27 && L.nr == 0 ? k_matvec<true> : k_matvec<false>, L.nblk, NT, 0, st,
+             L.view<double>(), x, y);
   }
   SSAMG_LAUNCH_CHECK();
 }
