@@ -1824,9 +1824,7 @@ bool brick_level(const Level& L) {
 }
 
 // Whether the operator applies of precision T run over bricks: where the tile
-// table says so and on large levels (beyond L2 each x is to be read once: 64
-// uneven problems, 72M cells, FP32 residual 403 us over bricks, 722 over tiles),
-// else by the rule.  A brick is one block marching 2048 cells,
+// table says so, else by the rule.  A brick is one block marching 2048 cells,
 // so a level needs enough of them, well filled; below that the cell tiles
 // spread it further.  The fill is by the bricks' time (brick_march): the bricks
 // of parts of a few planes end early, so that many tiny parts beside a large one
@@ -1843,10 +1841,23 @@ bool brick_level(const Level& L) {
 //   FP32 residual, last relaxation: 32^3 3.0, 5.8 / 1.5, 3.3; 8 x 33^3 (400, 0.41)
 //     6.6, 12.6 / 3.9, 7.8; 80^3 (300, 0.83) 4.0, 11.7 / 4.2, 7.3; 8 x 48^3 7.6, 13.0
 //     / 6.8, 13.3; 100^3 5.9, 12.9 / 6.7, 12.7; 8 x 64^3 9.9, 24.5 / 14.2, 35.6
+// Levels of SSAMG_K7_LARGE cells and more have bricks enough and take a lower fill
+// (by brick_march; bricks / tiles):
+//   FP64: a PCG iteration over bricks loses below 0.85 here too, 12 of 80^3 (0.83) 1312 /
+//     1280 us, 44 of 77^3 (0.77) 3966 / 3847, 20 of 67 x 64 x 64 (0.70) 1284 / 1192, 600 of
+//     9 x 32 x 32 (0.28) 1938 / 1283, but the solve of a batch gains, half the blocks left
+//     idle by the problems that have stopped: 64 problems x 4 right-hand sides (72M
+//     cells, 0.80) 1096 / 1152 ms, 40 problems (19M, 0.75) 78.3 / 82.1 (single problems
+//     between 0.75 and 0.85 pay 1 to 3 % for it)
+//   FP32 residual, last relaxation: 100 of 38^3 (0.56) 30.5, 77 / 34.9, 83 us; 1600 of 15^3
+//     (0.43) 40.3, 102 / 41.6, 89; 600 of 9 x 32 x 32 61, 151 / 36, 79; the 64 problems' solve
+//     606 / 724 ms
 template <class T>
 bool uses_bricks(const Level& L) {
   if (!brick_level(L)) return false;
-  if (L.bricks == 2 || L.N >= SSAMG_K7_LARGE) return true;
+  if (L.bricks == 2) return true;
+  if (L.N >= SSAMG_K7_LARGE)
+    return L.brick_march >= (sizeof(T) == 8 ? SSAMG_K7_FILL_LARGE_F64 : SSAMG_K7_FILL_LARGE_F32);
   return sizeof(T) == 8 ? L.nbblk >= SSAMG_K7_BRICKS_F64 && L.brick_march >= SSAMG_K7_FILL_F64
                         : L.nbblk >= SSAMG_K7_BRICKS_F32 && L.brick_march >= SSAMG_K7_FILL_F32;
 }

@@ -52,11 +52,13 @@
 #define SSAMG_BRICK_RESIDENT_FINAL32 5  // last relaxation
 // Fewest bricks of a level, and the least of Level::brick_march, for the operator
 // applies over bricks (see uses_bricks)
-#define SSAMG_K7_LARGE 5000000  // levels of this many cells always take them
 #define SSAMG_K7_BRICKS_F32 250
 #define SSAMG_K7_FILL_F32 0.6
 #define SSAMG_K7_BRICKS_F64 800
 #define SSAMG_K7_FILL_F64 0.85
+#define SSAMG_K7_LARGE 5000000  // the least fill from this many cells on
+#define SSAMG_K7_FILL_LARGE_F32 0.5
+#define SSAMG_K7_FILL_LARGE_F64 0.75
 #define SSAMG_DG_CELLS (152 * 256)  // smaller boxes (a block an SM) take dL/dg with a thread per cell
 #define SSAMG_DG_FILL 0.47  // and boxes that fill less of the shared-face form's 32 x 8 columns
 #define SSAMG_RP_BRICKS 152  // fewest bricks for the restriction / prolongation brick forms
