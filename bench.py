@@ -43,8 +43,8 @@ WORKLOAD = "8 parts x 64^3 (2x2x2 layout), 7-pt anisotropic diffusion, seed 1"
 L2_BYTES = 129 * 2 ** 20
 # FP64 peak of one GB300: 152 SMs x 2 FP64 FMA per clock per SM x 2 flops x 2.07 GHz
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# FP64-pipe instructions per cell of dL/dg: exp(g) (counted by ncu), then three
-# faces of 9, two products a face, kappa^2 and the result (counted in the source)
+# FP64-pipe instructions per cell of dL/dg, counted by ncu on the 128^3 case: exp(g),
+# then three faces of 9, two products a face, kappa^2 and the result
 FP64_INSTS_PER_CELL_DG = 15 + 39
 
 

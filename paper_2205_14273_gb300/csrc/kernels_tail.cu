@@ -28,9 +28,9 @@
 // side, is formed at setup as a dense matrix (one block per column runs that
 // sub-cycle on a unit vector) and applied like the coarsest inverse, one
 // barrier and 65,536 multiply-adds over the cluster.
-// Measured (tail of one cycle): 13 levels of one part, FP64 61.6 -> 26.7 us;
-// 10 levels of 8 parts, FP64 59 -> 37 us, FP32 38.4 -> 26 us; 13 levels of two
-// parts, FP32 43 -> 29 us.  A row's arithmetic is a small part of a step: four
+// Measured (tail of one cycle, replayed alone): 13 levels of one part, FP64 61.6 ->
+// 25.4 us, FP32 39.4 -> 25.2; 10 levels of 8 parts, FP64 55.4 -> 32.4, FP32 34.6 -> 26.0;
+// 13 levels of two parts, FP64 64.4 -> 31.3, FP32 43.6 -> 29.9 us.  A row's arithmetic is a small part of a step: four
 // barriers of ~0.3-0.5 us and a remote round trip remain per cluster level.
 #include <cooperative_groups.h>
 
